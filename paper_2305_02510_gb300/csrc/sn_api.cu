@@ -78,6 +78,109 @@ sn_status size_sparse_executor(sn_ctx *c) {
     return SN_OK;
 }
 
+// The pull store on the device: the entries, each slice's first uint4, the
+// region lengths of each position's list, and the positions.
+sn_status upload_pull_store(sn_ctx *c, const std::vector<uint4> &pin, const std::vector<long long> &off,
+                            const std::vector<int> &lens, const std::vector<int> &perm) {
+    const int n = c->n;
+    const size_t slices = off.size(), bytes = pin.size() * 16;
+    sn_status s;
+    if (c->pin && c->pin_cap < bytes) { dfree(c, c->pin); c->pin = nullptr; }
+    if (!c->pin) {
+        if ((s = dalloc(c, &c->pin, bytes))) return s;
+        c->pin_cap = bytes;
+    }
+    if (!c->pin_off) {
+        if ((s = dalloc(c, &c->pin_off, slices * 8)) || (s = dalloc(c, &c->pin_len, (size_t)n * 20)) ||
+            (s = dalloc(c, &c->pin_y0, (size_t)n * 8)) || (s = dalloc(c, &c->pin_perm, (size_t)n * 4)))
+            return s;
+    }
+    SN_CUDA(c, cudaMemcpy(c->pin, pin.data(), bytes, cudaMemcpyHostToDevice));
+    SN_CUDA(c, cudaMemcpy(c->pin_off, off.data(), slices * 8, cudaMemcpyHostToDevice));
+    SN_CUDA(c, cudaMemcpy(c->pin_len, lens.data(), lens.size() * 4, cudaMemcpyHostToDevice));
+    SN_CUDA(c, cudaMemcpy(c->pin_perm, perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice));
+    c->pin_bytes = (long long)bytes;
+    return SN_OK;
+}
+
+// The store of the blocked kernel (sn_pull_block.cu), from the CSR positions
+// `byd` in list order: five regions by delay per slice of 32 positions, each
+// padded to the slice's longest list.  Within each block's neurons the lists
+// are sorted by the first region (the longest work), then within runs of
+// three warps by the delay-1 region (on the step's critical path, and walked
+// three times as often).  Not built (pin_blocked stays false) for lists the
+// kernel cannot count or sum.
+sn_status build_block_store(sn_ctx *c, const std::vector<uint2> &syn, const std::vector<uint32_t> &byd,
+                            const std::vector<uint32_t> &pre_of) {
+    constexpr int kRegions = 5;
+    const int n = c->n, hb = c->pull_hb, slices = (n + 31) / 32;
+    const long long m = c->m;
+    c->pin_blocked = false;
+    auto region_of = [&](uint32_t p) {
+        const int d = (int)(syn[p].x >> kPostBits) + 1;
+        return d >= 7 ? 0 : d >= 4 ? 1 : 5 - d;
+    };
+    std::vector<int> len(kRegions * (size_t)n, 0);
+    for (long long k = 0; k < m; ++k) len[(size_t)region_of(byd[k]) * n + (syn[byd[k]].x & kPostMask)]++;
+    // the kernel counts a region's pairs in 16 bits and sums integers in 32
+    for (const int q : len)
+        if (q > 2 * 65535) return SN_OK;
+    if (c->dtype == SN_I32) {
+        std::vector<long long> sum(n, 0);
+        for (long long k = 0; k < m; ++k) sum[syn[k].x & kPostMask] += std::llabs((long long)(int)syn[k].y);
+        for (const long long q : sum)
+            if (q > 2147483647ll) return SN_OK;
+    }
+    std::vector<int> perm(n), pos_of(n);
+    for (int j = 0; j < n; ++j) perm[j] = j;
+    auto by_region = [&](int r) {
+        return [&len, n, r](int x, int y) { return len[(size_t)r * n + x] > len[(size_t)r * n + y]; };
+    };
+    for (int b0 = 0; b0 < n; b0 += c->pull_chunk) {
+        const int b1 = std::min(n, b0 + c->pull_chunk);
+        std::stable_sort(perm.begin() + b0, perm.begin() + b1, by_region(0));
+        for (int w0 = b0; w0 < b1; w0 += 96)
+            std::stable_sort(perm.begin() + w0, perm.begin() + std::min(b1, w0 + 96), by_region(4));
+    }
+    for (int q = 0; q < n; ++q) pos_of[perm[q]] = q;
+    std::vector<long long> off(slices), start(kRegions * (size_t)slices);
+    std::vector<int> lens(kRegions * (size_t)n);
+    long long total = 0;
+    for (int sl = 0; sl < slices; ++sl) {
+        off[sl] = total;
+        for (int r = 0; r < kRegions; ++r) {
+            int longest = 0;
+            for (int q = sl * 32; q < std::min(n, sl * 32 + 32); ++q) {
+                lens[(size_t)r * n + q] = len[(size_t)r * n + perm[q]];
+                longest = std::max(longest, lens[(size_t)r * n + q]);
+            }
+            start[(size_t)r * slices + sl] = total;
+            total += (long long)((longest + 1) / 2) * 32;
+        }
+    }
+    std::vector<uint4> pin(std::max(total, 1ll), make_uint4(0, 0, 0, 0));
+    std::fill(len.begin(), len.end(), 0);                // entries placed so far
+    std::vector<unsigned> word_at(n);
+    for (int i = 0; i < n; ++i) word_at[i] = pull_hist_byte((unsigned)i, hb) << 5;
+    for (long long k = 0; k < m; ++k) {
+        const uint32_t p = byd[k], pre = pre_of[p];
+        const int d = (int)(syn[p].x >> kPostBits) + 1, r = region_of(p), j = (int)(syn[p].x & kPostMask);
+        const int ps = pos_of[j], q = len[(size_t)r * n + j]++;
+        const unsigned x = r == 0 ? word_at[pre] | (unsigned)(d - 7)
+                         : r == 1 ? word_at[pre] | (unsigned)(d - 4) : (pre >> 5) << 7 | (pre & 31u);
+        uint4 &u = pin[start[(size_t)r * slices + (ps >> 5)] + (long long)(q >> 1) * 32 + (ps & 31)];
+        if (q & 1) { u.z = x; u.w = syn[p].y; } else { u.x = x; u.y = syn[p].y; }
+    }
+    sn_status s;
+    if (!c->ptag && (s = dalloc(c, &c->ptag, pull_tag_bytes(c->words)))) return s;
+    if ((s = upload_pull_store(c, pin, off, lens, perm))) return s;
+    c->pin_coded = 0;
+    c->pin_blocked = true;
+    c->pin_entries = m;
+    c->pin_stale = false;
+    return SN_OK;
+}
+
 // Incoming synapses of every neuron in the canonical order of the float sum:
 // descending delay, then ascending pre and input index (the oldest spikes
 // first), laid out for the pull kernel in two regions per slice of 32 neurons
@@ -126,6 +229,14 @@ sn_status build_pull_store(sn_ctx *c) {
             byd[dstart[D - 1 - (int)(syn[p].x >> kPostBits)]++] = (uint32_t)p;
             pre_of[p] = (uint32_t)i;
         }
+    // The blocked kernel, unless the coded form is asked for, also where its
+    // store outgrows the L2: it reads a synapse 0.44 times a step (10^5 neurons,
+    // delays 1..16, 100 steps: 110 synapses a neuron 0.89 ms against 1.09 of
+    // the best other form, 125: 1.04 against 1.22, 150 (147 MB): 1.19 against 1.50).
+    if (c->pull_hb && c->pin_format != 2) {
+        const sn_status st = build_block_store(c, syn, byd, pre_of);
+        if (st || c->pin_blocked) return st;
+    }
     const bool one_region = c->pull_grid == 1;
     const unsigned long long wbits = (unsigned long long)((c->words + 3) & ~3) * 32;   // window row, bits
     auto region_of = [&](uint32_t p) { return ((syn[p].x >> kPostBits) == 0 && !one_region) ? 1 : 0; };
@@ -224,39 +335,23 @@ sn_status build_pull_store(sn_ctx *c) {
             step -= 65535u;                               // a filler: weight 0
         }
     }
-    sn_status s;
-    const size_t bytes = (size_t)tot * 16;
-    if (c->pin && c->pin_cap < bytes) { dfree(c, c->pin); c->pin = nullptr; }
-    if (!c->pin) {
-        if ((s = dalloc(c, &c->pin, bytes))) return s;
-        c->pin_cap = bytes;
-    }
-    if (!c->pin_off) {
-        if ((s = dalloc(c, &c->pin_off, (size_t)slices * 8)) || (s = dalloc(c, &c->pin_len, (size_t)n * 4)) ||
-            (s = dalloc(c, &c->pin_len1, (size_t)n * 4)) || (s = dalloc(c, &c->pin_y0, (size_t)n * 8)) ||
-            (s = dalloc(c, &c->pin_perm, (size_t)n * 4)))
-            return s;
-    }
     // list lengths and first offsets by position
-    std::vector<int> lA(n), lB(n);
+    std::vector<int> lens(2 * (size_t)n);
     std::vector<unsigned> y0p(2 * (size_t)n);
     for (int q = 0; q < n; ++q) {
         const int j = perm[q];
-        lA[q] = (f ? lenc[0] : len[0])[j];
-        lB[q] = (f ? lenc[1] : len[1])[j];
-        y0p[q] = y0[j];
-        y0p[(size_t)n + q] = y0[(size_t)n + j];
+        for (int r = 0; r < 2; ++r) {
+            lens[(size_t)r * n + q] = (f ? lenc[r] : len[r])[j];
+            y0p[(size_t)r * n + q] = y0[(size_t)r * n + j];
+        }
     }
-    SN_CUDA(c, cudaMemcpy(c->pin, pin.data(), bytes, cudaMemcpyHostToDevice));
-    SN_CUDA(c, cudaMemcpy(c->pin_off, off[f].data(), (size_t)slices * 8, cudaMemcpyHostToDevice));
-    SN_CUDA(c, cudaMemcpy(c->pin_len, lA.data(), (size_t)n * 4, cudaMemcpyHostToDevice));
-    SN_CUDA(c, cudaMemcpy(c->pin_len1, lB.data(), (size_t)n * 4, cudaMemcpyHostToDevice));
+    sn_status s = upload_pull_store(c, pin, off[f], lens, perm);
+    if (s) return s;
     SN_CUDA(c, cudaMemcpy(c->pin_y0, y0p.data(), (size_t)n * 8, cudaMemcpyHostToDevice));
-    SN_CUDA(c, cudaMemcpy(c->pin_perm, perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice));
     c->pin_coded = f;
-    c->pin_bytes = (long long)bytes;
+    c->pin_blocked = false;
     c->pin_entries = 0;
-    for (int j = 0; j < n; ++j) c->pin_entries += (long long)lA[j] + lB[j];
+    for (const int q : lens) c->pin_entries += q;
     c->pin_stale = false;
     return SN_OK;
 }
@@ -273,6 +368,12 @@ sn_status select_pull(sn_ctx *c) {
                         "memory and at most 1024 neurons per SM");
     }
     sn_status s;
+    // a shard's rows come from other processes: one step at a time (sn_pull.cu)
+    if (!c->shard_end) {
+        cudaError_t e = plan_pull_block(c->n, c->D, c->dtype, c->pull_grid, c->pull_chunk, &c->pull_hb,
+                                        &c->pull_block_smem);
+        if (e != cudaSuccess) return cuda_fail(c, e, "blocked pull executor");
+    }
     if ((s = quiesce(c))) return s;            // a queued push run may still read the ring
     if (!c->hist) {
         if ((s = dalloc(c, &c->hist, (size_t)c->D * c->words * 4))) return s;
@@ -830,14 +931,15 @@ sn_status sn_run(sn_ctx *c, int32_t steps) {
             sn_status st = build_pull_store(c);
             if (st) return st;
         }
-        a.pin = c->pin; a.pin_off = c->pin_off; a.pin_len = c->pin_len; a.pin_len1 = c->pin_len1;
+        a.pin = c->pin; a.pin_off = c->pin_off; a.pin_len = c->pin_len; a.ptag = c->ptag;
         a.pin_y0 = c->pin_y0; a.pin_perm = c->pin_perm;
         a.ring_until = (int)std::min<long long>(c->ring_live_until, 2147483647ll);
         a.hL = c->pull_rows;
         a.chunk = c->pull_chunk;
         a.j_first = c->shard_end ? c->shard_first : 0;
         a.j_end = c->shard_end ? c->shard_end : c->n;
-        e = launch_sparse_pull(a, c->dtype, c->pin_coded != 0, c->pull_grid, c->pull_smem, c->stream);
+        e = c->pin_blocked ? launch_pull_block(a, c->dtype, c->pull_hb, c->pull_grid, c->pull_block_smem, c->stream)
+                           : launch_sparse_pull(a, c->dtype, c->pin_coded != 0, c->pull_grid, c->pull_smem, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "simulation launch");
         c->hist_live = true;
     } else {

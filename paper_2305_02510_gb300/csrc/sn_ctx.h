@@ -39,14 +39,17 @@ struct sn_ctx {
     size_t pull_smem = 0;
     uint4 *pin = nullptr;              // incoming synapses in 32-neuron slices
     long long *pin_off = nullptr;
-    int *pin_len = nullptr;            // entries of delay >= 2 of each thread position's list
-    int *pin_len1 = nullptr;           // entries of delay 1 of each thread position's list
+    int *pin_len = nullptr;            // [5][n] entries of each region of each thread position's list
     unsigned *pin_y0 = nullptr;        // coded store: [2][n] bit offset of each region's first entry
     int *pin_perm = nullptr;           // [n] the neuron whose lists thread position p sums
     size_t pin_cap = 0;                // bytes allocated for pin
     int pin_coded = 0;                 // 1: the store holds 16-bit offset steps (coded form)
     int pin_format = 0;                // 0 = the smaller of the two forms, 1 = plain, 2 = coded
     long long pin_bytes = 0, pin_entries = 0;   // store size; entries incl. padding and gap fillers
+    int pull_hb = 0;                   // blocked pull: bits of a neuron's spike word (0: does not fit)
+    size_t pull_block_smem = 0;
+    bool pin_blocked = false;          // the store is laid out for blocked pull (sn_pull_block.cu)
+    unsigned long long *ptag = nullptr;
     bool pin_stale = true;             // the pull store must be (re)built from the CSR
     unsigned *hist = nullptr;          // [D][words] spike bits whose deliveries may be due
     bool hist_live = false;            // hist may hold spikes not yet delivered

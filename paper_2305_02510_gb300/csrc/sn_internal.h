@@ -70,11 +70,15 @@ struct NetArgs {
     // (groups of 8 weights and 16-bit offset steps)
     const uint4 *pin;
     const long long *pin_off;         // [slices] first uint4 of each slice
-    const int *pin_len;               // [n] entries of delay >= 2 of each position's list
-    const int *pin_len1;              // [n] entries of delay 1 (the region after them)
+    const int *pin_len;               // [regions][n] entries of each region of each position's list
+                                      // (sn_pull.cu: delay >= 2, delay 1; sn_pull_block.cu: five)
     const unsigned *pin_y0;           // coded store: [2][n] window bit offset of each region's first entry
     const int *pin_perm;              // [n] the neuron whose lists thread position p sums (the store,
-                                      // pin_len, pin_len1 and pin_y0 are indexed by position)
+                                      // pin_len and pin_y0 are indexed by position)
+    unsigned long long *ptag;         // blocked pull: spike words of the last steps with the step's
+                                      // number in the high half (sn_pull_block.cu)
+    int wp, wt, rows_at, acc_at;     // blocked pull: words rounded up to 4 and to 2, bytes of shared
+                                      // memory before the two rows and before the sums
     unsigned *hist;                   // [hD][words] spike bits of step tau in row tau % hD
     int hD;                           // history depth (the maximum delay D)
     int hL;                           // rows of the pull kernel's shared-memory window
@@ -223,6 +227,11 @@ cudaError_t plan_pull(int n, int D, long long m, int *grid, int *chunk, int *row
 cudaError_t launch_shard_put(unsigned *hist, unsigned *raster, int D, int cap, int words, int w0, int w1,
                              long long t0, int rows, const unsigned *src, cudaStream_t s);
 cudaError_t launch_sparse_pull(const NetArgs &a, int dtype, bool coded, int grid, size_t smem, cudaStream_t s);
+// Pull in blocks of three steps (sn_pull_block.cu).
+cudaError_t plan_pull_block(int n, int D, int dtype, int grid, int chunk, int *hb, size_t *smem);
+size_t pull_tag_bytes(int words);
+unsigned pull_hist_byte(unsigned pre, int hb);
+cudaError_t launch_pull_block(NetArgs a, int dtype, int hb, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_pull_flush(const NetArgs &a, int dtype, int t0, cudaStream_t s);
 cudaError_t launch_gather_weights(const uint2 *syn, const long long *perm_inv, long long m,
                                   float *out, cudaStream_t s);

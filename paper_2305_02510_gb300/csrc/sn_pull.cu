@@ -2,6 +2,8 @@
 // timestep: the input of neuron j is the sum over its incoming synapses of
 // w * s_i(t - d); Section 2.2: a spike reaches the post-neuron d steps later).
 //
+// This kernel takes one step at a time: networks of one block, shards, the
+// coded store, and networks whose spike words do not fit sn_pull_block.cu.
 // Every block keeps the spike bits of recent steps in a shared-memory window
 // of hL rows of Wp = roundup(ceil(n/32), 4) words: the row of step tau sits
 // at position tau - base.  Each thread owns one neuron and holds its state in
@@ -45,22 +47,12 @@
 #include <algorithm>
 
 #include "sn_device.cuh"
+#include "sn_pull.cuh"
 
 namespace sn {
 namespace {
 
 constexpr int kPullUnroll = 4;      // 16-byte loads (two synapses each) per half of the double buffer
-constexpr int kPullMaxBlock = 1024;
-
-template <int MODE> struct PullAcc;
-template <> struct PullAcc<SN_F32> {
-    using T = float;
-    static __device__ __forceinline__ T add(T acc, unsigned wbits) { return __fadd_rn(acc, __uint_as_float(wbits)); }
-};
-template <> struct PullAcc<SN_I32> {
-    using T = long long;            // exact: int32 weights, at most 2^32 synapses
-    static __device__ __forceinline__ T add(T acc, unsigned wbits) { return acc + (long long)(int)wbits; }
-};
 
 // One synapse: the bit of its pre-neuron at step t - d, from the window whose
 // first row (step t - D) starts at byte `row0` of shared memory.
@@ -94,13 +86,11 @@ __device__ __forceinline__ void pull_batch_part(typename PullAcc<MODE>::T &acc, 
         }
     }
 }
-
 __device__ __forceinline__ void pull_load(uint4 (&e)[kPullUnroll], const uint4 *ent, int p0, int np) {
 #pragma unroll
     for (int u = 0; u < kPullUnroll; ++u)
         e[u] = p0 + u < np ? __ldg(ent + (size_t)(p0 + u) * 32) : make_uint4(0u, 0u, 0u, 0u);
 }
-
 
 // Coded store: a group of 8 synapses is three uint4s of a lane (weights 0-3,
 // weights 4-7, eight 16-bit offset steps), 96 uint4s apart per group in a
@@ -244,7 +234,7 @@ __global__ void __launch_bounds__(kPullMaxBlock, 1) sparse_pull_kernel(NetArgs a
         amp = ((const V *)a.pamp)[j];
         // units of the store per region: pairs (plain) or groups of 8 (coded)
         npA = CODED ? (a.pin_len[j] + 7) >> 3 : (a.pin_len[j] + 1) >> 1;
-        npB = CODED ? (a.pin_len1[j] + 7) >> 3 : (a.pin_len1[j] + 1) >> 1;
+        npB = CODED ? (a.pin_len[(size_t)a.n + j] + 7) >> 3 : (a.pin_len[(size_t)a.n + j] + 1) >> 1;
         if (CODED) {
             yA = a.pin_y0[j];
             yB = a.pin_y0[(size_t)a.n + j];
