@@ -255,6 +255,9 @@ __global__ void __launch_bounds__(kPullMaxBlock, 1) sparse_pull_kernel(NetArgs a
     uint4 ea[CODED ? kCodedBuf : kPullUnroll], eb[CODED ? kCodedBuf : kPullUnroll];
     region_start(ea, ent, npA);
     __syncthreads();
+    // the slot of row t0 - D is the first to be stored again: not before every
+    // block has read it
+    if (gridDim.x > 1 && !grid_barrier(a.ctl)) return;
     // the delay >= 2 part of the first step: every row it reads is in the window
     Acc acc = 0;
     if (a.steps > 0) {
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__(kPullMaxBlock, 1) sparse_pull_kernel(NetArgs a
         // grid barrier, split: arrive, do this block's independent work, wait
         __syncthreads();                              // every warp's words of step t are stored
         unsigned gen = 0;
-        if (threadIdx.x == 0 && gridDim.x > 1) gen = bar_arrive_k(a.ctl, (unsigned)s);
+        if (threadIdx.x == 0 && gridDim.x > 1) gen = bar_arrive_k(a.ctl, (unsigned)s + 1u);
         // a single block reads the status word now, so that the read overlaps
         // the work below (a grid reads it after the barrier)
         int stop_early = 0;
