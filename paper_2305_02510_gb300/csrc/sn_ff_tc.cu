@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constan
     const uint32_t tmem = s_tmem;
     constexpr uint32_t idesc = idesc_bf16_f32(kT, kT);
     unsigned g_prod = 0, g_mma = 0, items_done = 0;
+    bool ready = false;                            // the next stage's operands are known to be there
     const int items = a.tiles_m * a.tiles_n * a.ksplit;
 
     for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
@@ -110,8 +111,10 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constan
                         tma_load_2d(dA + 2 * kStageA, &maps.m[ps.bmap2], ps.b_x + kb * kKB, ps.b_y2 + tn * kT, fb);
                 }
             }
-        } else if (warp == 1 && lane == 0) {
-            // MMA issuer; an accumulator's first MMA of this item overwrites it
+        } else if (warp == 1) {
+            // MMA issuer; an accumulator's first MMA of this item overwrites it.
+            // The next stage's barrier is looked at before this stage's MMAs are
+            // issued.
             int started = 0;
             for (int p = 0; p < a.npass && !s_abort; ++p) {
                 const FfTcPass &ps = a.pass[p];
@@ -121,22 +124,26 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constan
                 for (int kb = kb0; kb < kb1; ++kb, ++g_mma) {
                     const int st = g_mma % kSt;
                     const unsigned round = g_mma / kSt;
-                    if (!mbar_wait(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
+                    if (!ready && !mbar_wait(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
+                    ready = mbar_test(smem_addr(&full[(g_mma + 1) % kSt]), ((g_mma + 1) / kSt) & 1u);
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint32_t dA = sbase + st * kStageBytes;
-                    for (int q = 0; q < ps.nb; ++q) {
+                    const int on = (started >> ps.acc) & 1;
 #pragma unroll
-                        for (int kk = 0; kk < 128 / 32; ++kk) {
-                            const int on = ((started >> ps.acc) & 1) | (q > 0) | (kk > 0);
-                            mma_bf16(tacc, umma_desc_sw128(dA + kk * 32),
-                                     umma_desc_sw128(dA + (1 + q) * kStageA + kk * 32), idesc, on);
-                        }
+                    for (int kk = 0; kk < 128 / 32; ++kk)
+                        mma_bf16(tacc, umma_desc_sw128(dA + kk * 32), umma_desc_sw128(dA + kStageA + kk * 32), idesc,
+                                 on | (kk > 0));
+                    if (ps.nb > 1) {
+#pragma unroll
+                        for (int kk = 0; kk < 128 / 32; ++kk)
+                            mma_bf16(tacc, umma_desc_sw128(dA + kk * 32), umma_desc_sw128(dA + 2 * kStageA + kk * 32),
+                                     idesc, 1);
                     }
-                    started |= 1 << ps.acc;
                     mma_commit(smem_addr(&empty[st]));
+                    started |= 1 << ps.acc;
                 }
             }
-            s_started = started;
+            if (lane == 0) s_started = started;
             mma_commit(smem_addr(&accbar));
         }
         __syncwarp();
@@ -290,7 +297,8 @@ __global__ void __launch_bounds__(kFwdTcThreads, 1) ff_tc_fwd_kernel(const __gri
                                     ps.b_y + q * a.part_stride + tn * kT, fb);
                 }
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        bool ready = false;                        // the next stage's operands are known to be there
         unsigned g_chunk = 0;
         for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x)
             for (int kb = 0; kb < KB && !s_abort; ++kb, ++g_chunk) {
@@ -301,7 +309,8 @@ __global__ void __launch_bounds__(kFwdTcThreads, 1) ff_tc_fwd_kernel(const __gri
                 for (int p = 0; p < a.npass; ++p, ++g_mma) {
                     const int st = g_mma % kFwdSt;
                     const unsigned round = g_mma / kFwdSt;
-                    if (!mbar_wait(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
+                    if (!ready && !mbar_wait(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
+                    ready = mbar_test(smem_addr(&full[(g_mma + 1) % kFwdSt]), ((g_mma + 1) / kFwdSt) & 1u);
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint32_t dA = sbase + st * kFwdStageBytes;
 #pragma unroll

@@ -158,7 +158,7 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
                     tma_load_2d(dA, tmA, kb * kTK, m0, fb);
                     tma_load_2d(dA + kStageA, &tmW, kb * kTK, n0, fb);
                 }
-            } else if (warp == 1 && lane == 0) {
+            } else if (warp == 1) {
                 // MMA issuer
                 for (int kb = 0; kb < kblocks; ++kb, ++g_mma) {
                     const int st = g_mma % kStages;
