@@ -973,8 +973,12 @@ sn_status sn_reset(sn_ctx *c) {
         const size_t bn = (size_t)c->sh_B * c->n;
         SN_CUDA(c, cudaMemcpyAsync(c->V, c->sh_V0, bn * 4, cudaMemcpyDeviceToDevice, c->stream));
         SN_CUDA(c, cudaMemsetAsync(c->r, 0, bn * 4, c->stream));
-        SN_CUDA(c, cudaMemsetAsync(c->sh_A0, 0, bn, c->stream));
-        SN_CUDA(c, cudaMemsetAsync(c->sh_A1, 0, bn, c->stream));
+        if (c->sh_res) {
+            SN_CUDA(c, cudaMemsetAsync(c->sh_bits, 0, bn / 32 * 2 * 8, c->stream));
+        } else {
+            SN_CUDA(c, cudaMemsetAsync(c->sh_A0, 0, bn, c->stream));
+            SN_CUDA(c, cudaMemsetAsync(c->sh_A1, 0, bn, c->stream));
+        }
         SN_CUDA(c, cudaMemsetAsync(c->raster, 0, (size_t)c->cap * c->words * 4, c->stream));
         SN_CUDA(c, cudaMemsetAsync(c->ctl, 0, sizeof(Control), c->stream));
         c->step = 0;
@@ -1256,8 +1260,8 @@ sn_status sn_save(sn_ctx *c, void *buf, size_t *size) {
     cudaError_t e;
     if (c->kind == KIND_SHARED_I8) {
         const size_t bn = (size_t)c->sh_B * c->n;
-        if ((e = get(c->V, bn * 4)) || (e = get(c->r, bn * 4)) || (e = get(c->sh_A0, bn)) || (e = get(c->sh_A1, bn)))
-            return cuda_fail(c, e, "save");
+        if ((e = get(c->V, bn * 4)) || (e = get(c->r, bn * 4))) return cuda_fail(c, e, "save");
+        if ((st = shared_save_spikes(c, p))) return st;
         *size = need;
         return SN_OK;
     }
@@ -1301,8 +1305,8 @@ sn_status sn_load(sn_ctx *c, const void *buf, size_t size) {
     cudaError_t e;
     if (c->kind == KIND_SHARED_I8) {
         const size_t bn = (size_t)c->sh_B * c->n;
-        if ((e = put(c->V, bn * 4)) || (e = put(c->r, bn * 4)) || (e = put(c->sh_A0, bn)) || (e = put(c->sh_A1, bn)))
-            return cuda_fail(c, e, "load");
+        if ((e = put(c->V, bn * 4)) || (e = put(c->r, bn * 4))) return cuda_fail(c, e, "load");
+        if ((s = shared_load_spikes(c, p))) return s;
     } else {
         if ((e = put(c->V, (size_t)c->n * 4)) || (e = put(c->r, (size_t)c->n * 4)) ||
             (e = put(c->ring, c->ring_bytes)))

@@ -119,6 +119,8 @@ struct sn_ctx {
     // shared dense network driven by many trains (tensor cores)
     int sh_B = 0, sh_grid = 0;
     unsigned char *sh_A0 = nullptr, *sh_A1 = nullptr, *sh_WT = nullptr;
+    int sh_res = 0;                    // 1: one tile per block (sn_shared_res.cu), spikes in sh_bits
+    unsigned long long *sh_bits = nullptr;
     int *sh_V0 = nullptr;
     alignas(64) unsigned char sh_tmaps[3 * 128];
     // shard of a sparse network (sn_create_shard): neurons [shard_first,
@@ -235,6 +237,8 @@ void destroy_all(sn_ctx *c);
 sn_status batch_run(sn_ctx *c, int steps);
 sn_status sparse_autotune(sn_ctx *c, int trial_steps, float *best_ms);
 sn_status shared_run(sn_ctx *c, int steps);
+sn_status shared_save_spikes(sn_ctx *c, uint8_t *out);
+sn_status shared_load_spikes(sn_ctx *c, const uint8_t *in);
 sn_status shared_get_state(sn_ctx *c, void *v, int32_t *refr, int32_t on_device);
 sn_status shared_set_poisson(sn_ctx *c, int32_t nsrc, const int32_t *neuron, const float *rate,
                              const float *amp, uint64_t seed, uint64_t net0);

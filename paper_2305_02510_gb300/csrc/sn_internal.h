@@ -139,7 +139,8 @@ cudaError_t batch_kernel_node(int dtype, void **fn);
 cudaError_t max_grid_batch(int dtype, int ring_smem, int *grid);
 size_t batch_smem(int ring_smem);
 
-// Shared dense network on tensor cores, sn_shared.cu
+// Shared dense network on tensor cores: sn_shared.cu, and sn_shared_res.cu when
+// every block holds one tile (spikes as tagged bit words instead of A0, A1)
 struct SharedHostArgs {
     int n, B, t0, steps, cap;
     unsigned char *A0, *A1;
@@ -149,8 +150,12 @@ struct SharedHostArgs {
     const int *pamp;
     const unsigned long long *pkey;
     unsigned *raster;
+    unsigned long long *bits;
     Control *ctl;
 };
+cudaError_t plan_shared_res(int n, int B, int *fits);
+cudaError_t launch_shared_res(const void *tmap_w, const SharedHostArgs &h, cudaStream_t s);
+int wt_res_pos(int i);
 cudaError_t launch_shared(const void *tmaps, const SharedHostArgs &h, int grid, cudaStream_t s);
 cudaError_t max_grid_shared(int *grid);
 size_t shared_smem_bytes();

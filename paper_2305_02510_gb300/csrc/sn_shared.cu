@@ -17,11 +17,9 @@
 // and stage the tile's neuron parameters in shared memory.  Afterwards the
 // sixteen warps read the accumulator rows (tcgen05.ld: warps w, w+4, w+8 and
 // w+12 share TMEM lane quarter w, each taking 32 columns) and apply the integer LIF
-// rule (Section 2.1 order).  When every block holds one tile for the whole
-// launch (tiles <= blocks), the tile's V and r stay in TMEM next to the
-// accumulator (columns 128.. and 256..), read from global memory at the
-// launch's start and written back at its end; otherwise they make the round
-// trip every step.  The global state is neuron-major ([n][B]: lane = train,
+// rule (Section 2.1 order).  This form serves networks of more tiles than blocks
+// (sn_shared_res.cu: one tile per block for the whole launch); the state makes
+// the round trip through global memory every step.  The global state is neuron-major ([n][B]: lane = train,
 // so every load and store of V and r is one 128-byte line per warp); the
 // spike bytes that are the next step's A operand go through a shared-memory
 // transpose and leave as whole 128-byte rows.  A persistent cooperative
@@ -35,13 +33,11 @@
 
 #include "sn_device.cuh"
 #include "sn_internal.h"
+#include "sn_shared.cuh"
 #include "sn_tc.cuh"
 
 namespace sn {
 
-constexpr int kTM = 128;                       // trains per tile (MMA M)
-constexpr int kTN = 128;                       // post-neurons per tile (MMA N)
-constexpr int kTK = 128;                       // bytes of K per stage (one 128B swizzle row)
 constexpr int kStages = 6;
 constexpr int kStageA = kTM * kTK;             // 16 KiB
 constexpr int kStageBytes = (kTM + kTN) * kTK; // 32 KiB
@@ -55,26 +51,7 @@ constexpr int kSub = 4;                      // state columns loaded together
 constexpr int kSaPitch = 144;                  // 128 B + 16: conflict-free 16-byte stores
 constexpr int kEpiBytes = kTM * kSaPitch + 2 * kTM * 4 * 4 + 5 * kTN * 4;
 constexpr unsigned kTmemCols = 128;
-// When every block holds one tile for the whole launch, the tile's state
-// stays in TMEM between steps: V at columns kVCol + c, r at kRCol + c of the
-// train's lane (512 columns allocated: the accumulator's 128 and 256 of state).
-constexpr unsigned kTmemColsRes = 512;
-constexpr uint32_t kVCol = 128, kRCol = 256;
 
-struct SharedArgs {
-    int n, B, t0, steps, cap, words;
-    int tiles_m, tiles;
-    unsigned char *A0, *A1;        // spike operands [B][n] bytes, A_(t & 1) holds step t
-    int *V, *r;                    // [n][B] (neuron-major)
-    const int *th, *lk, *rs, *R;   // [n]
-    const unsigned *prate;         // [n]
-    const int *pamp;               // [n]
-    const unsigned long long *pkey;// [B]
-    unsigned *raster;              // [cap][B][words]
-    Control *ctl;
-};
-
-template <bool kRes>
 __global__ void __launch_bounds__(kShThreads, 1)
 shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
               const __grid_constant__ CUtensorMap tmW, SharedArgs a) {
@@ -101,7 +78,7 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         s_abort = 0;
     }
-    constexpr unsigned kCols = kRes ? kTmemColsRes : kTmemCols;
+    constexpr unsigned kCols = kTmemCols;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
                      :: "r"(smem_addr(&s_tmem)), "r"(kCols));
@@ -114,22 +91,6 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
     const int quarter = warp & 3, part = warp >> 2;
     const int bl = quarter * 32 + lane;                // tile row = TMEM lane
     const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);   // this warp's lane quarter
-    if (kRes && blockIdx.x < a.tiles) {
-        // the block's one tile: its state into TMEM for the whole launch
-        const int m0 = (blockIdx.x % a.tiles_m) * kTM, n0 = (blockIdx.x / a.tiles_m) * kTN;
-        for (int h = 0; h < kEpiCols / 16; ++h) {
-            const int c0 = part * kEpiCols + h * 16;
-            const int *Vp = a.V + (size_t)(n0 + c0) * a.B + m0 + bl;
-            const int *rp = a.r + (size_t)(n0 + c0) * a.B + m0 + bl;
-            uint32_t vv[16], rr[16];
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                vv[q] = (uint32_t)__ldcg(Vp + (size_t)q * a.B);
-                rr[q] = (uint32_t)__ldcg(rp + (size_t)q * a.B);
-            }
-            tmem_st16x2(trow + kVCol + c0, trow + kRCol + c0, vv, rr);
-        }
-    }
     const int kblocks = a.n / kTK;
     constexpr uint32_t idesc = idesc_e4m3_f32(kTM, kTN);
     unsigned g_prod = 0, g_mma = 0, tiles_done = 0;
@@ -208,39 +169,7 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
                 const unsigned pb = sP[bl * 4 + (c0 >> 5)];
                 unsigned bits = 0;
                 uint32_t outw[8];
-                if constexpr (kRes) {
-                    // accumulator and state from TMEM, state back, 16
-                    // columns at a time (the stores run even after a failed
-                    // wait: tcgen05.st is warp-collective)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint32_t col = (uint32_t)(c0 + 16 * h);
-                        uint32_t v[16], vv[16], rr[16];
-                        tmem_ld16x3(trow + col, trow + kVCol + col, trow + kRCol + col, v, vv, rr);
-                        if (ok) {
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {
-                                uint32_t bytes = 0;
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    const int qq = q4 * 4 + e, q = h * 16 + qq, c = c0 + q;
-                                    const int acc = __float2int_rn(__uint_as_float(v[qq]));
-                                    const int ext = ((pb >> q) & 1u) ? sAmp[c] : 0;
-                                    int vq = (int)vv[qq], rq = (int)rr[qq];
-                                    const bool fire = lif_update_i32(vq, rq, acc, ext, sTh[c], sLk[c], sRs[c],
-                                                                     sRf[c], overflow);
-                                    vv[qq] = (uint32_t)vq;
-                                    rr[qq] = (uint32_t)rq;
-                                    bits |= (unsigned)fire << q;
-                                    bytes |= (fire ? 0x38u : 0u) << (8 * e);      // E4M3 1.0
-                                }
-                                outw[h * 4 + q4] = bytes;
-                            }
-                        }
-                        tmem_st16x2(trow + kVCol + col, trow + kRCol + col, vv, rr);
-                    }
-                    if (!ok) continue;
-                } else {
+                {
                     uint32_t v[32];
                     tmem_ld32(trow + (uint32_t)c0, v);
                     if (!ok) continue;
@@ -324,25 +253,6 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (kRes && blockIdx.x < a.tiles) {
-        // the tile's state back to its neuron-major arrays
-        const int m0 = (blockIdx.x % a.tiles_m) * kTM, n0 = (blockIdx.x / a.tiles_m) * kTN;
-        for (int h = 0; h < kEpiCols / 16; ++h) {
-            const int c0 = part * kEpiCols + h * 16;
-            int *Vp = a.V + (size_t)(n0 + c0) * a.B + m0 + bl;
-            int *rp = a.r + (size_t)(n0 + c0) * a.B + m0 + bl;
-            uint32_t vv[16], rr[16];
-            tmem_ld16x2(trow + kVCol + c0, trow + kRCol + c0, vv, rr);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                __stcg(Vp + (size_t)q * a.B, (int)vv[q]);
-                __stcg(rp + (size_t)q * a.B, (int)rr[q]);
-            }
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    }
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(kCols));
     if (overflow) atomicCAS(&a.ctl->status, 0, (int)SN_EOVERFLOW);
     if (my_spikes) {
@@ -373,12 +283,10 @@ cudaError_t max_grid_shared(int *grid) {
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    for (const void *f : {(const void *)shared_kernel<false>, (const void *)shared_kernel<true>}) {
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared_smem_bytes());
-        if (e != cudaSuccess) return e;
-    }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, (const void *)shared_kernel<false>, kShThreads,
-                                                      shared_smem_bytes());
+    const void *f = (const void *)shared_kernel;
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared_smem_bytes());
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, kShThreads, shared_smem_bytes());
     if (e != cudaSuccess) return e;
     // one block per SM: TMEM columns and the 128 KiB pipeline are per block
     *grid = (per > 0 ? 1 : 0) * sms;
@@ -386,21 +294,14 @@ cudaError_t max_grid_shared(int *grid) {
 }
 
 cudaError_t launch_shared(const void *tmaps, const SharedHostArgs &h, int grid, cudaStream_t s) {
-    SharedArgs a;
-    a.n = h.n; a.B = h.B; a.t0 = h.t0; a.steps = h.steps; a.cap = h.cap; a.words = h.n / 32;
-    a.tiles_m = h.B / kTM;
-    a.tiles = a.tiles_m * (h.n / kTN);
-    a.A0 = h.A0; a.A1 = h.A1; a.V = h.V; a.r = h.r;
-    a.th = h.th; a.lk = h.lk; a.rs = h.rs; a.R = h.R;
-    a.prate = h.prate; a.pamp = h.pamp; a.pkey = h.pkey; a.raster = h.raster; a.ctl = h.ctl;
+    const SharedArgs a = shared_args(h);
     const CUtensorMap *tm = (const CUtensorMap *)tmaps;
     const int g = grid < a.tiles ? grid : a.tiles;
     void *args[] = {(void *)&tm[0], (void *)&tm[1], (void *)&tm[2], (void *)&a};
     // the grid barrier's arrival count starts every launch at zero
     cudaError_t e = cudaMemsetAsync(&h.ctl->bar, 0, sizeof(GridBarrier), s);
     if (e != cudaSuccess) return e;
-    // one tile per block for the whole launch: the state stays in TMEM
-    const void *f = g == a.tiles ? (const void *)shared_kernel<true> : (const void *)shared_kernel<false>;
+    const void *f = (const void *)shared_kernel;
     return cudaLaunchCooperativeKernel(f, dim3(g), dim3(kShThreads), args, shared_smem_bytes(), s);
 }
 

@@ -44,13 +44,51 @@ static sn_status encode_map(sn_ctx *c, EncodeTiled fn, void *out, void *base, lo
     return SN_OK;
 }
 
+// The two spike operands as a checkpoint holds them: E4M3 bytes [trains][n] of
+// the last even and the last odd step.
+static size_t shared_word_at(const sn_ctx *c, size_t q) {
+    // word q of [2][trains][n / 32] in the kernel's order, [2][n / 128][trains][4]
+    const size_t w = c->n / 32, B = c->sh_B, part = q / (B * w), b = q / w % B, k = q % w;
+    return ((part * (w / 4) + k / 4) * B + b) * 4 + k % 4;
+}
+
+sn_status shared_save_spikes(sn_ctx *c, uint8_t *out) {
+    const size_t bn = (size_t)c->sh_B * c->n;
+    if (!c->sh_res) {
+        SN_CUDA(c, cudaMemcpy(out, c->sh_A0, bn, cudaMemcpyDeviceToHost));
+        SN_CUDA(c, cudaMemcpy(out + bn, c->sh_A1, bn, cudaMemcpyDeviceToHost));
+        return SN_OK;
+    }
+    std::vector<unsigned long long> w(bn / 32 * 2);
+    SN_CUDA(c, cudaMemcpy(w.data(), c->sh_bits, w.size() * 8, cudaMemcpyDeviceToHost));
+    for (size_t q = 0; q < w.size(); ++q)
+        for (int i = 0; i < 32; ++i) out[q * 32 + i] = (w[shared_word_at(c, q)] >> i) & 1 ? 0x38 : 0;
+    return SN_OK;
+}
+
+sn_status shared_load_spikes(sn_ctx *c, const uint8_t *in) {
+    const size_t bn = (size_t)c->sh_B * c->n;
+    if (!c->sh_res) {
+        SN_CUDA(c, cudaMemcpy(c->sh_A0, in, bn, cudaMemcpyHostToDevice));
+        SN_CUDA(c, cudaMemcpy(c->sh_A1, in + bn, bn, cudaMemcpyHostToDevice));
+        return SN_OK;
+    }
+    std::vector<unsigned long long> w(bn / 32 * 2, 0ull);
+    for (size_t q = 0; q < w.size(); ++q)
+        for (int i = 0; i < 32; ++i) w[shared_word_at(c, q)] |= (unsigned long long)(in[q * 32 + i] != 0) << i;
+    SN_CUDA(c, cudaMemcpy(c->sh_bits, w.data(), w.size() * 8, cudaMemcpyHostToDevice));
+    return SN_OK;
+}
+
 sn_status shared_run(sn_ctx *c, int steps) {
     SharedHostArgs h;
     h.n = c->n; h.B = c->sh_B; h.t0 = (int)c->step; h.steps = steps; h.cap = c->cap;
     h.A0 = c->sh_A0; h.A1 = c->sh_A1; h.V = (int *)c->V; h.r = c->r;
     h.th = (const int *)c->th; h.lk = (const int *)c->lk; h.rs = (const int *)c->rs; h.R = c->R;
-    h.prate = c->prate; h.pamp = (const int *)c->pamp; h.pkey = c->pkeys; h.raster = c->raster; h.ctl = c->ctl;
-    cudaError_t e = launch_shared(c->sh_tmaps, h, c->sh_grid, c->stream);
+    h.prate = c->prate; h.pamp = (const int *)c->pamp; h.pkey = c->pkeys; h.raster = c->raster; h.bits = c->sh_bits;
+    h.ctl = c->ctl;
+    cudaError_t e = c->sh_res ? launch_shared_res(c->sh_tmaps + 256, h, c->stream)
+                              : launch_shared(c->sh_tmaps, h, c->sh_grid, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "shared dense launch");
     return SN_OK;
 }
@@ -136,8 +174,18 @@ extern "C" sn_status sn_create_shared_dense_i8(const sn_config *cfg, const sn_ne
     c->words = (int)(bn / 32);
     c->cap = cfg->record_steps > 0 ? cfg->record_steps : 1;
     int *V = nullptr, *r = nullptr;
+    {
+        cudaError_t e = plan_shared_res(n, trains, &c->sh_res);
+        if (e != cudaSuccess) {
+            c->err = std::string("shared dense occupancy: ") + cudaGetErrorString(e);
+            return bail(SN_EUNSUPPORTED);
+        }
+    }
+    if (c->sh_res ? (s = dalloc(c, &c->sh_bits, bn / 32 * 2 * 8))
+                  : (s = dalloc(c, &c->sh_A0, bn)) || (s = dalloc(c, &c->sh_A1, bn)))
+        return bail(s);
     if ((s = dalloc(c, &V, bn * 4)) || (s = dalloc(c, &r, bn * 4)) || (s = dalloc(c, &c->sh_V0, bn * 4)) ||
-        (s = dalloc(c, &c->sh_A0, bn)) || (s = dalloc(c, &c->sh_A1, bn)) || (s = dalloc(c, &c->sh_WT, nn)) ||
+        (s = dalloc(c, &c->sh_WT, nn)) ||
         (s = dalloc(c, &c->pkeys, (size_t)trains * 8)) ||
         (s = dalloc(c, &c->raster, (size_t)c->cap * c->words * 4)) || (s = dalloc(c, &c->ctl, sizeof(Control))))
         return bail(s);
@@ -149,7 +197,8 @@ extern "C" sn_status sn_create_shared_dense_i8(const sn_config *cfg, const sn_ne
         uint8_t lut[17];
         for (int v = -8; v <= 8; ++v) lut[v + 8] = e4m3_of_int(v);
         for (int i = 0; i < n; ++i)
-            for (int j = 0; j < n; ++j) wt[(size_t)j * n + i] = lut[w[(size_t)i * n + j] + 8];
+            for (int j = 0, at = c->sh_res ? wt_res_pos(i) : i; j < n; ++j)
+                wt[(size_t)j * n + at] = lut[w[(size_t)i * n + j] + 8];
         // the kernel keeps the state neuron-major, [n][trains]
         std::vector<int> v0(bn);
         for (int j = 0; j < n; ++j)
@@ -160,7 +209,9 @@ extern "C" sn_status sn_create_shared_dense_i8(const sn_config *cfg, const sn_ne
         if ((e = cudaMemcpy(c->sh_WT, wt.data(), nn, cudaMemcpyHostToDevice)) ||
             (e = cudaMemcpy(c->sh_V0, v0.data(), bn * 4, cudaMemcpyHostToDevice)) ||
             (e = cudaMemcpy(c->V, v0.data(), bn * 4, cudaMemcpyHostToDevice)) ||
-            (e = cudaMemset(c->r, 0, bn * 4)) || (e = cudaMemset(c->sh_A0, 0, bn)) || (e = cudaMemset(c->sh_A1, 0, bn)) ||
+            (e = cudaMemset(c->r, 0, bn * 4)) ||
+            (e = c->sh_res ? cudaMemset(c->sh_bits, 0, bn / 32 * 2 * 8) : cudaMemset(c->sh_A0, 0, bn)) ||
+            (e = c->sh_res ? cudaSuccess : cudaMemset(c->sh_A1, 0, bn)) ||
             (e = cudaMemcpy(c->pkeys, keys.data(), (size_t)trains * 8, cudaMemcpyHostToDevice)) ||
             (e = cudaMemset(c->raster, 0, (size_t)c->cap * c->words * 4)) || (e = cudaMemset(c->ctl, 0, sizeof(Control)))) {
             c->err = std::string("upload: ") + cudaGetErrorString(e);
@@ -174,8 +225,8 @@ extern "C" sn_status sn_create_shared_dense_i8(const sn_config *cfg, const sn_ne
         c->err = "cuTensorMapEncodeTiled is not available from the driver";
         return bail(SN_EUNSUPPORTED);
     }
-    if ((s = encode_map(c, (EncodeTiled)fn, c->sh_tmaps + 0, c->sh_A0, trains, n)) ||
-        (s = encode_map(c, (EncodeTiled)fn, c->sh_tmaps + 128, c->sh_A1, trains, n)) ||
+    if ((!c->sh_res && ((s = encode_map(c, (EncodeTiled)fn, c->sh_tmaps + 0, c->sh_A0, trains, n)) ||
+                        (s = encode_map(c, (EncodeTiled)fn, c->sh_tmaps + 128, c->sh_A1, trains, n)))) ||
         (s = encode_map(c, (EncodeTiled)fn, c->sh_tmaps + 256, c->sh_WT, n, n)))
         return bail(s);
     cudaError_t e = max_grid_shared(&c->sh_grid);

@@ -93,6 +93,25 @@ __device__ __forceinline__ void mma_f8(uint32_t tmem, uint64_t adesc, uint64_t b
         :: "r"(tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
 }
 
+// The four MMAs of a 128-byte K block with A in tensor memory (row = lane, four
+// 8-bit elements of K per 32-bit column: an MMA of K = 32 takes 8 columns), and
+// the commits of the block's two operand stages, under one election.
+__device__ __forceinline__ void mma_f8_block_ta(uint32_t tmem, uint32_t ta, uint64_t bdesc, uint32_t idesc, int acc,
+                                                uint32_t bar_a, uint32_t bar_b) {
+    asm volatile(
+        "{\n.reg .pred p, q, t;\n.reg .b32 a1, a2, a3;\n.reg .b64 b1, b2, b3;\n"
+        "elect.sync _|q, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\nsetp.eq.u32 t, 0, 0;\n"
+        "add.u32 a1, %1, 8;\nadd.u32 a2, %1, 16;\nadd.u32 a3, %1, 24;\n"
+        "add.u64 b1, %2, 2;\nadd.u64 b2, %2, 4;\nadd.u64 b3, %2, 6;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [a1], b1, %3, t;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [a2], b2, %3, t;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [a3], b3, %3, t;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n}\n"
+        :: "r"(tmem), "r"(ta), "l"(bdesc), "r"(idesc), "r"(acc), "r"(bar_a), "r"(bar_b) : "memory");
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\n"
                  "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n"
@@ -132,25 +151,29 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, uint32_t (
         : "memory");
 }
 
-// Three 16-column TMEM loads and the wait for all three.
-__device__ __forceinline__ void tmem_ld16x3(uint32_t ta, uint32_t tb, uint32_t tc, uint32_t (&a)[16],
-                                            uint32_t (&b)[16], uint32_t (&c)[16]) {
+// Three 8-column TMEM loads and the wait for all three.
+__device__ __forceinline__ void tmem_ld8x3(uint32_t ta, uint32_t tb, uint32_t tc, uint32_t (&a)[8], uint32_t (&b)[8],
+                                           uint32_t (&c)[8]) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%48];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%49];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47}, [%50];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%24];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%25];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%26];\n"
         "tcgen05.wait::ld.sync.aligned;\n"
         : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]),
-          "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]),
-          "=r"(a[15]), "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]),
-          "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]), "=r"(b[11]), "=r"(b[12]), "=r"(b[13]),
-          "=r"(b[14]), "=r"(b[15]), "=r"(c[0]), "=r"(c[1]), "=r"(c[2]), "=r"(c[3]), "=r"(c[4]), "=r"(c[5]),
-          "=r"(c[6]), "=r"(c[7]), "=r"(c[8]), "=r"(c[9]), "=r"(c[10]), "=r"(c[11]), "=r"(c[12]),
-          "=r"(c[13]), "=r"(c[14]), "=r"(c[15])
+          "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7]),
+          "=r"(c[0]), "=r"(c[1]), "=r"(c[2]), "=r"(c[3]), "=r"(c[4]), "=r"(c[5]), "=r"(c[6]), "=r"(c[7])
         : "r"(ta), "r"(tb), "r"(tc)
+        : "memory");
+}
+
+// Two 8-column TMEM stores and the wait for both.
+__device__ __forceinline__ void tmem_st8x2(uint32_t ta, uint32_t tb, const uint32_t (&a)[8], const uint32_t (&b)[8]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%2,%3,%4,%5,%6,%7,%8,%9};\n"
+        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%1], {%10,%11,%12,%13,%14,%15,%16,%17};\n"
+        "tcgen05.wait::st.sync.aligned;\n"
+        :: "r"(ta), "r"(tb), "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]),
+           "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]), "r"(b[7])
         : "memory");
 }
 
@@ -171,6 +194,18 @@ __device__ __forceinline__ void tmem_st16x2(uint32_t ta, uint32_t tb, const uint
            "r"(b[15])
         : "memory");
 }
+
+// A 16-column TMEM store (this warp's lane quarter); tmem_st_wait waits for the
+// stores issued before it.
+__device__ __forceinline__ void tmem_st16(uint32_t ta, const uint32_t (&a)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
+        :: "r"(ta), "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]),
+           "r"(a[8]), "r"(a[9]), "r"(a[10]), "r"(a[11]), "r"(a[12]), "r"(a[13]), "r"(a[14]), "r"(a[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 
 // Instruction descriptor of kind::f16 with BF16 A and B, FP32 accumulator,
 // both K-major.
