@@ -113,7 +113,9 @@ struct sn_ctx {
     int ff_engine = 0;                 // SN_FF_AUTO, SN_FF_SIMT or SN_FF_TENSOR
     bool ff_tc_ok = false;             // the shapes fit the tensor-core path
     bool ff_fwd_tc = false;            // the last forward ran on the tensor cores
-    void *ff_Sbf = nullptr, *ff_ST = nullptr, *ff_G = nullptr, *ff_GT = nullptr;
+    std::vector<void *> ff_Sbf;        // spikes of layers 0 .. L-1 (one buffer for all: ff_S_shared)
+    bool ff_S_shared = false;
+    void *ff_G = nullptr;
     std::vector<void *> ff_Wf, ff_Wb;  // forward and backward weight parts per layer
     void *ff_encode = nullptr;         // the driver's cuTensorMapEncodeTiled
     // shared dense network driven by many trains (tensor cores)

@@ -23,6 +23,7 @@
 // contractions; sn_ff_tc.cu holds their tensor-core forms, which the host
 // code uses by default (sn_ff_set_engine).
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -239,7 +240,7 @@ template <int K>
 __global__ void __launch_bounds__(kBwdBlock) ff_scan_bwd_kernel(const float *__restrict__ I, int n, int B, int T,
                                    FFNeuron p, const float *__restrict__ vck, const int *__restrict__ rck,
                                    const float *__restrict__ gs, const float *__restrict__ gc,
-                                   float *__restrict__ gI) {
+                                   float *__restrict__ gI, __nv_bfloat16 *__restrict__ gbf, int ldg) {
     __shared__ float sI[2][K][kBwdBlock], sG[2][K][kBwdBlock];
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (tid >= (long long)B * n) return;
@@ -312,7 +313,15 @@ __global__ void __launch_bounds__(kBwdBlock) ff_scan_bwd_kernel(const float *__r
             const float sur = mk[q] ? __frcp_rn(__fmul_rn(den, den)) : 0.0f;
             const float g = Gb ? sG[buf][q][threadIdx.x] : gcount;
             const float gu = (sp[q] ? 0.0f : gv) + g * sur;
-            gIb[(size_t)t * stride] = gu;
+            if (gbf) {
+                // the two parts of the tensor cores' operand: hi + mid
+                __nv_bfloat16 *g2 = gbf + (size_t)(t * B + b) * ldg + j;
+                const __nv_bfloat16 hi = __float2bfloat16_rn(gu);
+                *g2 = hi;
+                g2[(size_t)T * B * ldg] = __float2bfloat16_rn(__fsub_rn(gu, __bfloat162float(hi)));
+            } else {
+                gIb[(size_t)t * stride] = gu;
+            }
             const float dv = vprev[q] - p.reset;
             gv = (fabsf(dv) > p.leak) ? gu : 0.0f;
         }
@@ -554,16 +563,17 @@ cudaError_t ff_scan_fwd(const float *I, int n, int B, int T, int k, float theta,
 
 cudaError_t ff_scan_bwd(const float *I, int n, int B, int T, int k, float theta, float leak, float reset,
                         int refractory, float slope, const float *vck, const int *rck, const float *gs,
-                        const float *gc, float *gI, cudaStream_t s) {
+                        const float *gc, float *gI, void *gbf, int ldg, cudaStream_t s) {
     FFNeuron p{theta, leak, reset, slope, refractory};
     const long long threads = (long long)B * n;
     const int nb = blocks_for(threads, kBwdBlock);
+    __nv_bfloat16 *g2 = (__nv_bfloat16 *)gbf;
     switch (k) {
-        case 1: ff_scan_bwd_kernel<1><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI); break;
-        case 2: ff_scan_bwd_kernel<2><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI); break;
-        case 5: ff_scan_bwd_kernel<5><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI); break;
-        case 10: ff_scan_bwd_kernel<10><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI); break;
-        case 20: ff_scan_bwd_kernel<20><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI); break;
+        case 1: ff_scan_bwd_kernel<1><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
+        case 2: ff_scan_bwd_kernel<2><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
+        case 5: ff_scan_bwd_kernel<5><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
+        case 10: ff_scan_bwd_kernel<10><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
+        case 20: ff_scan_bwd_kernel<20><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -22,12 +22,12 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 
 inline int up(int x, int m) { return (x + m - 1) / m * m; }
 
-// Row-major BF16 [rows][cols] (cols a multiple of 64), boxes of 128 rows x 64
+// Row-major BF16 [rows][cols] (cols a multiple of 64), boxes of box_rows rows x 64
 // columns, 128-byte swizzle; coordinates outside the tensor read as zero.
-sn_status bf16_map(sn_ctx *c, CUtensorMap *out, const void *base, long long rows, long long cols) {
+sn_status bf16_map(sn_ctx *c, CUtensorMap *out, const void *base, long long rows, long long cols, int box_rows = 128) {
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    cuuint32_t box[2] = {64, 128};
+    cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     cuuint32_t es[2] = {1, 1};
     CUresult r = ((EncodeTiledFn)c->ff_encode)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)base, dims, strides,
                                                box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -40,23 +40,18 @@ bool use_tc(const sn_ctx *c) { return c->ff_tc_ok && c->ff_engine != SN_FF_SIMT;
 
 // Synaptic input of layer l for all rows, I[r][j] = sum_d sum_i S[r - dB][i] W_d[i][j]:
 // 4 delays x 3 exact BF16 weight parts (4 passes of 3 parts each), accumulated
-// block by block (ff_tc_forward).  Unpacks the previous layer's spikes, and their transpose
-// when the weight gradient will need it.
-sn_status tc_forward(sn_ctx *c, int l, bool want_st, float *I, bool sbf_ready = false) {
+// block by block (ff_tc_forward), from the spike operand of layer l - 1.
+sn_status tc_forward(sn_ctx *c, int l, float *I) {
     const int B = c->ff_batch, rows = B * c->ff_steps;
     const int nin = c->ff_sizes[l - 1], nout = c->ff_sizes[l];
-    const int nin_p = up(nin, 64), rows_out = up(nout, 128), rows_p = up(rows, 64);
-    cudaError_t e = cudaSuccess;
-    if (!sbf_ready || want_st)
-        e = ff_tc_spikes(c->ff_S[l - 1], rows, nin, (nin + 31) / 32, nin_p, rows_p, sbf_ready ? nullptr : c->ff_Sbf,
-                         want_st ? c->ff_ST : nullptr, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "spike operands");
+    const int nin_p = up(nin, 64), rows_out = up(nout, 128);
+    cudaError_t e;
     FfTcMaps maps;
     FfTcArgs a;
     memset(&maps, 0, sizeof(maps));
     memset(&a, 0, sizeof(a));
     sn_status s;
-    if ((s = bf16_map(c, &maps.m[0], c->ff_Sbf, rows, nin_p)) ||
+    if ((s = bf16_map(c, &maps.m[0], c->ff_Sbf[l - 1], rows, nin_p)) ||
         (s = bf16_map(c, &maps.m[1], c->ff_Wf[l - 1], 12LL * rows_out, nin_p)))
         return s;
     // one pass per delay; the kernel multiplies its spike tile by the three
@@ -65,59 +60,52 @@ sn_status tc_forward(sn_ctx *c, int l, bool want_st, float *I, bool sbf_ready = 
         FfTcPass &ps = a.pass[a.npass++];
         ps.amap = 0; ps.a_y = -d * B; ps.a_x = 0;
         ps.bmap = 1; ps.b_y = (d - 1) * 3 * rows_out; ps.b_x = 0;
-        ps.kblocks = nin_p / 64; ps.acc = 0;
+        ps.kblocks = nin_p / 64;
     }
     a.part_stride = rows_out;
     a.M = rows; a.N = nout;
-    a.tiles_m = (rows + 127) / 128; a.tiles_n = (nout + 127) / 128; a.ksplit = 1;
-    a.nacc = 1; a.mode = 0; a.C = I; a.ldc = nout; a.cstride = 0; a.ctl = c->ctl;
+    a.tiles_m = (rows + 127) / 128; a.tiles_n = (nout + 127) / 128;
+    a.C = I; a.ldc = nout; a.ctl = c->ctl;
     if ((e = ff_tc_forward(maps, a, c->stream)) != cudaSuccess) return cuda_fail(c, e, "tensor-core synaptic input");
     return SN_OK;
 }
 
-// Weight gradient of layer l from gI (already split and transposed into GT)
-// and the transposed spikes ST: 4 delays x 2 gradient parts, one accumulator
-// per delay, split over K (the rows) to fill the GPU, then reduced in order.
+// Weight gradient of layer l from the spike operand of layer l - 1 and the
+// gradient's parts G: four delays at once (ff_tc_dw), split over K (the rows) to
+// fill the GPU, then reduced in order.
 sn_status tc_weight_grad(sn_ctx *c, int l, float *dW) {
     const int B = c->ff_batch, rows = B * c->ff_steps;
     const int nin = c->ff_sizes[l - 1], nout = c->ff_sizes[l];
-    const int rows_p = up(rows, 64);
+    const int nout_p = up(nout, 64);
     FfTcMaps maps;
-    FfTcArgs a;
+    FfTcDwArgs a;
     memset(&maps, 0, sizeof(maps));
     memset(&a, 0, sizeof(a));
     sn_status s;
-    const __nv_bfloat16 *GT = (const __nv_bfloat16 *)c->ff_GT;
-    if ((s = bf16_map(c, &maps.m[0], c->ff_ST, nin, rows_p)) ||
-        (s = bf16_map(c, &maps.m[1], GT, nout, rows_p)) ||
-        (s = bf16_map(c, &maps.m[2], GT + (size_t)nout * rows_p, nout, rows_p)))
+    const __nv_bfloat16 *G = (const __nv_bfloat16 *)c->ff_G;
+    if ((s = bf16_map(c, &maps.m[0], c->ff_Sbf[l - 1], rows, up(nin, 64), 64)) ||
+        (s = bf16_map(c, &maps.m[1], G, rows, nout_p, 64)) ||
+        (s = bf16_map(c, &maps.m[2], G + (size_t)rows * nout_p, rows, nout_p, 64)))
         return s;
-    // one pass per delay: the shifted spike tile times both gradient parts
-    for (int d = 1; d <= 4; ++d) {
-        FfTcPass &ps = a.pass[a.npass++];
-        ps.amap = 0; ps.a_y = 0; ps.a_x = -d * B;
-        ps.bmap = 1; ps.b_y = 0; ps.b_x = 0;
-        ps.nb = 2; ps.bmap2 = 2; ps.b_y2 = 0;
-        ps.kblocks = rows_p / 64; ps.acc = d - 1;
-    }
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    a.M = nin; a.N = nout;
+    a.M = nin; a.N = nout; a.B = B;
     a.tiles_m = (nin + 127) / 128; a.tiles_n = (nout + 127) / 128;
+    a.kblocks = (rows + 63) / 64;
     const int tiles = a.tiles_m * a.tiles_n;
     // K (the T * B rows) split over enough blocks to fill the GPU, as far as
     // the partial-sum buffer holds the splits (a narrow output layer has few
     // tiles and takes many splits)
     const long long cap = (long long)(c->ff_part_elems / ((size_t)nin * nout));
-    int ks = (int)std::max(1LL, std::min<long long>({(long long)(sms / std::max(1, tiles)), cap,
-                                                     (long long)(rows_p / 64 / 8)}));
+    const int ks = (int)std::max(1LL, std::min<long long>({(long long)(sms / std::max(1, tiles)), cap,
+                                                           (long long)(a.kblocks / 8)}));
     a.ksplit = ks;
-    a.nacc = 4; a.mode = 1; a.D = c->ff_D[l - 1]; a.ldc = nout; a.ctl = c->ctl;
+    a.D = c->ff_D[l - 1]; a.ctl = c->ctl;
     const long long count = (long long)nin * nout;
     a.C = ks == 1 ? dW : c->ff_part;
     a.cstride = count;
-    cudaError_t e = ff_tc_gemm(maps, a, c->stream);
+    cudaError_t e = ff_tc_dw(maps, a, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core weight gradient");
     if (ks > 1 && (e = ff_dw_reduce(c->ff_part, ks, count, dW, c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "weight gradient reduction");
@@ -146,16 +134,16 @@ sn_status tc_spike_grad(sn_ctx *c, int l) {
         ps.amap = 0; ps.a_y = d * B; ps.a_x = 0;
         ps.bmap = 2; ps.b_y = (d - 1) * 2 * rows_in; ps.b_x = 0;
         ps.nb = 2; ps.bmap2 = 2; ps.b_y2 = ((d - 1) * 2 + 1) * rows_in;
-        ps.kblocks = nout_p / 64; ps.acc = 0;
+        ps.kblocks = nout_p / 64;
         FfTcPass &pl = a.pass[a.npass++];
         pl.amap = 1; pl.a_y = d * B; pl.a_x = 0;
         pl.bmap = 2; pl.b_y = (d - 1) * 2 * rows_in; pl.b_x = 0;
         pl.nb = 1;
-        pl.kblocks = nout_p / 64; pl.acc = 0;
+        pl.kblocks = nout_p / 64;
     }
     a.M = rows; a.N = nin;
-    a.tiles_m = (rows + 127) / 128; a.tiles_n = (nin + 127) / 128; a.ksplit = 1;
-    a.nacc = 1; a.mode = 0; a.C = c->ff_gS; a.ldc = nin; a.cstride = 0; a.ctl = c->ctl;
+    a.tiles_m = (rows + 127) / 128; a.tiles_n = (nin + 127) / 128;
+    a.C = c->ff_gS; a.ldc = nin; a.ctl = c->ctl;
     cudaError_t e = ff_tc_gemm(maps, a, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core spike gradient");
     return SN_OK;
@@ -165,23 +153,20 @@ sn_status tc_spike_grad(sn_ctx *c, int l) {
 // any failure the context keeps the SIMT engine only.
 void tc_setup(sn_ctx *c) {
     const int L = c->ff_layers, B = c->ff_batch, rows = B * c->ff_steps;
-    if (B % 8 != 0) return;                    // delay shifts of d * B rows must stay 16-byte aligned in K
+    if (B % 8 != 0) return;
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
         q != cudaDriverEntryPointSuccess || !fn)
         return;
     c->ff_encode = fn;
-    const int rows_p = up(rows, 64);
-    size_t s_elems = 0, st_elems = 0, g_elems = 0, gt_elems = 0;
+    size_t s_elems = 0, g_elems = 0;
     c->ff_Wf.assign(L, nullptr);
     c->ff_Wb.assign(L, nullptr);
     for (int l = 1; l <= L; ++l) {
         const int nin = c->ff_sizes[l - 1], nout = c->ff_sizes[l];
         s_elems = std::max(s_elems, (size_t)rows * up(nin, 64));
-        st_elems = std::max(st_elems, (size_t)nin * rows_p);
         g_elems = std::max(g_elems, (size_t)2 * rows * up(nout, 64));
-        gt_elems = std::max(gt_elems, (size_t)2 * nout * rows_p);
         const size_t wf = (size_t)12 * up(nout, 128) * up(nin, 64) * 2, wb = (size_t)8 * up(nin, 128) * up(nout, 64) * 2;
         if (dalloc(c, &c->ff_Wf[l - 1], wf) || dalloc(c, &c->ff_Wb[l - 1], wb))
             return;
@@ -190,15 +175,19 @@ void tc_setup(sn_ctx *c) {
         // weight's own delay slot)
         if (cudaMemset(c->ff_Wf[l - 1], 0, wf) || cudaMemset(c->ff_Wb[l - 1], 0, wb)) return;
     }
-    if (dalloc(c, &c->ff_Sbf, s_elems * 2) || dalloc(c, &c->ff_ST, st_elems * 2) || dalloc(c, &c->ff_G, g_elems * 2) ||
-        dalloc(c, &c->ff_GT, gt_elems * 2))
-        return;
-    // padding columns and rows of the operands stay zero from here on (the
-    // spike rows' padding may later hold 0/1 values of a wider layer, which
-    // meet zero weight columns)
-    if (cudaMemset(c->ff_Sbf, 0, s_elems * 2) || cudaMemset(c->ff_ST, 0, st_elems * 2) ||
-        cudaMemset(c->ff_G, 0, g_elems * 2) || cudaMemset(c->ff_GT, 0, gt_elems * 2))
-        return;
+    // The spike operand of every layer stays for the weight gradient, like the
+    // synaptic input; a context that recomputes that also expands the spikes
+    // again, into one buffer.
+    c->ff_S_shared = c->ff_Ik.empty();
+    c->ff_Sbf.assign(L, nullptr);
+    for (int l = 0; l < L; ++l) {
+        if (l > 0 && c->ff_S_shared) { c->ff_Sbf[l] = c->ff_Sbf[0]; continue; }
+        const size_t bytes = (c->ff_S_shared ? s_elems : (size_t)rows * up(c->ff_sizes[l], 64)) * 2;
+        // padding columns stay zero (in a shared buffer they may later hold 0/1
+        // values of a wider layer, which meet zero weight columns)
+        if (dalloc(c, &c->ff_Sbf[l], bytes) || cudaMemset(c->ff_Sbf[l], 0, bytes)) return;
+    }
+    if (dalloc(c, &c->ff_G, g_elems * 2) || cudaMemset(c->ff_G, 0, g_elems * 2)) return;
     c->ff_tc_ok = true;
 }
 
@@ -346,7 +335,7 @@ sn_status sn_ff_forward(sn_ctx *c, const uint8_t *input, const float *const *w, 
     // with the tensor cores, the input packing and each layer's recurrence
     // also write the spikes as the next contraction's BF16 operand
     cudaError_t e = ff_pack(input, rows, c->ff_sizes[0], (c->ff_sizes[0] + 31) / 32, c->ff_S[0],
-                            tc ? c->ff_Sbf : nullptr, up(c->ff_sizes[0], 64), c->stream);
+                            tc ? c->ff_Sbf[0] : nullptr, up(c->ff_sizes[0], 64), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "input pack");
     for (int l = 1; l <= L; ++l) {
         const int nin = c->ff_sizes[l - 1], nout = c->ff_sizes[l];
@@ -358,7 +347,7 @@ sn_status sn_ff_forward(sn_ctx *c, const uint8_t *input, const float *const *w, 
                                    l > 1 ? c->ff_Wb[l - 1] : nullptr, (nin + 63) / 64 * 64, (nout + 127) / 128 * 128,
                                    c->ff_Wf[l - 1], c->stream)))
                 return cuda_fail(c, e, "weight parts");
-            sn_status st = tc_forward(c, l, false, I, true);
+            sn_status st = tc_forward(c, l, I);
             if (st) return st;
         } else if ((e = ff_delay_fwd(c->ff_S[l - 1], (nin + 31) / 32, w[l - 1], c->ff_DM[l - 1], nin, nout, B, 0,
                                      rows, I, c->stream))) {
@@ -366,7 +355,7 @@ sn_status sn_ff_forward(sn_ctx *c, const uint8_t *input, const float *const *w, 
         }
         if ((e = ff_scan_fwd(I, nout, B, T, c->ff_k, c->ff_theta, c->ff_leak, c->ff_reset, c->ff_refr,
                              c->ff_S[l], c->ff_vck[l], c->ff_rck[l], l == L ? counts : nullptr,
-                             tc && l < L ? c->ff_Sbf : nullptr, up(nout, 64), c->stream)))
+                             tc && l < L ? c->ff_Sbf[l] : nullptr, up(nout, 64), c->stream)))
             return cuda_fail(c, e, "forward recurrence");
     }
     c->ff_have_forward = true;
@@ -390,16 +379,15 @@ sn_status sn_backward(sn_ctx *c, const float *grad_counts, float *const *grad_w,
         const int nin = c->ff_sizes[l - 1], nout = c->ff_sizes[l];
         const int words_in = (nin + 31) / 32;
         // the forward's synaptic input: kept, or recomputed with the
-        // forward's own kernel so that the states match; the tensor-core
-        // weight gradient also takes the transposed input spikes
+        // forward's own kernel so that the states match
         float *I = c->ff_I;
+        if (tc && c->ff_S_shared &&
+            (e = ff_tc_spikes(c->ff_S[l - 1], rows, nin, words_in, up(nin, 64), c->ff_Sbf[l - 1], c->stream)))
+            return cuda_fail(c, e, "spike operands");
         if (!c->ff_Ik.empty()) {
             I = c->ff_Ik[l];
-            if (tc && (e = ff_tc_spikes(c->ff_S[l - 1], rows, nin, words_in, up(nin, 64), up(rows, 64), nullptr,
-                                        c->ff_ST, c->stream)))
-                return cuda_fail(c, e, "spike operands");
         } else if (tc) {
-            sn_status st = tc_forward(c, l, true, I);
+            sn_status st = tc_forward(c, l, I);
             if (st) return st;
         } else if ((e = ff_delay_fwd(c->ff_S[l - 1], words_in, c->ff_w[l - 1], c->ff_DM[l - 1], nin, nout, B, 0,
                                      rows, I, c->stream))) {
@@ -407,13 +395,10 @@ sn_status sn_backward(sn_ctx *c, const float *grad_counts, float *const *grad_w,
         }
         if ((e = ff_scan_bwd(I, nout, B, T, c->ff_k, c->ff_theta, c->ff_leak, c->ff_reset, c->ff_refr,
                              c->ff_slope, c->ff_vck[l], c->ff_rck[l], l == L ? nullptr : c->ff_gS,
-                             l == L ? grad_counts : nullptr, c->ff_gI, c->stream)))
+                             l == L ? grad_counts : nullptr, c->ff_gI, tc ? c->ff_G : nullptr, up(nout, 64),
+                             c->stream)))
             return cuda_fail(c, e, "adjoint recurrence");
         if (tc) {
-            const int nout_p = (nout + 63) / 64 * 64, rows_p = (rows + 63) / 64 * 64;
-            if ((e = ff_tc_gsplit(c->ff_gI, rows, nout, nout_p, rows_p, l > 1 ? c->ff_G : nullptr, c->ff_GT,
-                                  c->stream)))
-                return cuda_fail(c, e, "gradient parts");
             sn_status st = tc_weight_grad(c, l, grad_w[l - 1]);
             if (st) return st;
             if (l > 1 && (st = tc_spike_grad(c, l))) return st;

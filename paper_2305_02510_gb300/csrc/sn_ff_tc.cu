@@ -56,10 +56,10 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constan
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ __align__(8) uint64_t full[kSt], empty[kSt], accbar;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_abort, s_started;
+    __shared__ int s_abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sbase = smem_addr(smem);
-    const unsigned ncols = a.nacc <= 1 ? 128u : a.nacc == 2 ? 256u : 512u;
+    constexpr unsigned ncols = 128;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kSt; ++s) {
@@ -83,18 +83,15 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constan
     constexpr uint32_t idesc = idesc_bf16_f32(kT, kT);
     unsigned g_prod = 0, g_mma = 0, items_done = 0;
     bool ready = false;                            // the next stage's operands are known to be there
-    const int items = a.tiles_m * a.tiles_n * a.ksplit;
+    const int items = a.tiles_m * a.tiles_n;
 
     for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
-        const int ks = item % a.ksplit, tile = item / a.ksplit;
-        const int tm = tile % a.tiles_m, tn = tile / a.tiles_m;
+        const int tm = item % a.tiles_m, tn = item / a.tiles_m;
         if (warp == 0 && lane == 0) {
-            // TMA producer over every pass's K blocks of this split
+            // TMA producer over every pass's K blocks
             for (int p = 0; p < a.npass && !s_abort; ++p) {
                 const FfTcPass &ps = a.pass[p];
-                const int kb0 = (int)((long long)ps.kblocks * ks / a.ksplit);
-                const int kb1 = (int)((long long)ps.kblocks * (ks + 1) / a.ksplit);
-                for (int kb = kb0; kb < kb1; ++kb, ++g_prod) {
+                for (int kb = 0; kb < ps.kblocks; ++kb, ++g_prod) {
                     const int st = g_prod % kSt;
                     const unsigned round = g_prod / kSt;
                     if (round > 0 && !mbar_wait(smem_addr(&empty[st]), (round - 1) & 1u, a.ctl)) {
@@ -112,38 +109,32 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constan
                 }
             }
         } else if (warp == 1) {
-            // MMA issuer; an accumulator's first MMA of this item overwrites it.
-            // The next stage's barrier is looked at before this stage's MMAs are
-            // issued.
-            int started = 0;
+            // MMA issuer; the item's first MMA overwrites the accumulator.  The
+            // next stage's barrier is looked at before this stage's MMAs go out.
+            int on = 0;
             for (int p = 0; p < a.npass && !s_abort; ++p) {
                 const FfTcPass &ps = a.pass[p];
-                const int kb0 = (int)((long long)ps.kblocks * ks / a.ksplit);
-                const int kb1 = (int)((long long)ps.kblocks * (ks + 1) / a.ksplit);
-                const uint32_t tacc = tmem + (uint32_t)(ps.acc * kT);
-                for (int kb = kb0; kb < kb1; ++kb, ++g_mma) {
+                for (int kb = 0; kb < ps.kblocks; ++kb, ++g_mma) {
                     const int st = g_mma % kSt;
                     const unsigned round = g_mma / kSt;
                     if (!ready && !mbar_wait(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
                     ready = mbar_test(smem_addr(&full[(g_mma + 1) % kSt]), ((g_mma + 1) / kSt) & 1u);
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint32_t dA = sbase + st * kStageBytes;
-                    const int on = (started >> ps.acc) & 1;
 #pragma unroll
                     for (int kk = 0; kk < 128 / 32; ++kk)
-                        mma_bf16(tacc, umma_desc_sw128(dA + kk * 32), umma_desc_sw128(dA + kStageA + kk * 32), idesc,
+                        mma_bf16(tmem, umma_desc_sw128(dA + kk * 32), umma_desc_sw128(dA + kStageA + kk * 32), idesc,
                                  on | (kk > 0));
                     if (ps.nb > 1) {
 #pragma unroll
                         for (int kk = 0; kk < 128 / 32; ++kk)
-                            mma_bf16(tacc, umma_desc_sw128(dA + kk * 32), umma_desc_sw128(dA + 2 * kStageA + kk * 32),
+                            mma_bf16(tmem, umma_desc_sw128(dA + kk * 32), umma_desc_sw128(dA + 2 * kStageA + kk * 32),
                                      idesc, 1);
                     }
                     mma_commit(smem_addr(&empty[st]));
-                    started |= 1 << ps.acc;
+                    on = 1;
                 }
             }
-            if (lane == 0) s_started = started;
             mma_commit(smem_addr(&accbar));
         }
         __syncwarp();
@@ -157,38 +148,20 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constan
         // pipeline buffers, then leave as coalesced rows
         float *Cs = (float *)smem;                  // [128][kCPitch]
         const int quarter = warp & 3, half = warp >> 2;
-        const int ml = quarter * 32 + lane, m = tm * kT + ml;
-        const int started = s_started;
+        const int ml = quarter * 32 + lane;
         for (int cc = 0; cc < 2; ++cc) {
             const int c0 = half * 64 + cc * 32;
-            const int n0 = tn * kT + c0;
-            float out[32];
-#pragma unroll
-            for (int q = 0; q < 32; ++q) out[q] = 0.0f;
-            const int nacc = a.mode == 1 ? a.nacc : 1;
-            for (int d = 0; d < nacc; ++d) {
-                uint32_t v[32];
-                tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(d * kT + c0), v);
-                if (!ok || !((started >> d) & 1)) continue;
-                if (a.mode == 0) {
-#pragma unroll
-                    for (int q = 0; q < 32; ++q) out[q] = __uint_as_float(v[q]);
-                } else if (m < a.M) {
-                    // the weight gradient of (m, n) is that of its own delay
-                    const uint8_t *Dr = a.D + (size_t)m * a.N;
-#pragma unroll
-                    for (int q = 0; q < 32; ++q)
-                        if (n0 + q < a.N && Dr[n0 + q] == d + 1) out[q] = __uint_as_float(v[q]);
-                }
-            }
+            uint32_t v[32];
+            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
             float4 *dst = (float4 *)(Cs + ml * kCPitch + c0);
 #pragma unroll
             for (int q4 = 0; q4 < 8; ++q4)
-                dst[q4] = make_float4(out[4 * q4], out[4 * q4 + 1], out[4 * q4 + 2], out[4 * q4 + 3]);
+                dst[q4] = make_float4(__uint_as_float(v[4 * q4]), __uint_as_float(v[4 * q4 + 1]),
+                                      __uint_as_float(v[4 * q4 + 2]), __uint_as_float(v[4 * q4 + 3]));
         }
         __syncthreads();
         if (ok) {
-            float *C = a.C + (size_t)ks * a.cstride;
+            float *C = a.C;
             const int ncol = min(kT, a.N - tn * kT);
             for (int row = warp; row < kT; row += kThreads / 32) {
                 const int mm = tm * kT + row;
@@ -214,6 +187,163 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constan
     if (warp == 1 && lane == 0) {
         for (unsigned i = g_mma > kSt ? g_mma - kSt : 0; i < g_mma; ++i)
             mbar_wait(smem_addr(&empty[i % kSt]), (i / kSt) & 1u, a.ctl);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(ncols));
+}
+
+// Weight gradient: dW[i][j] = sum over the rows r of S[r - dB][i] gI[r][j], d the
+// synapse's own delay.  One 128 x 128 tile per work item with four TMEM
+// accumulators, one per delay; K is the rows, 64 a stage.  A stage holds the spike
+// tile shifted by each of the four delays and both parts of the gradient tile (96
+// KiB, 32 MMAs): the gradient is read once for the four delays (48 bytes a cycle
+// into the SM at the MMAs' full rate; one delay a stage took 94, which the L2
+// does not give).  Both operands are taken as they lie, rows of K with the inputs
+// or outputs contiguous (MN-major), so nothing is transposed for them.
+// 256 threads as in ff_tc_kernel.  12,800 rows: 1024 x 1024 183 -> 152 us, 700 x 1024
+// 130 -> 116 us, and the transposes (60 us) are gone.
+constexpr int kDwSt = 2;
+constexpr int kDwHalf = 64 * 128;               // 64 rows x 64 columns: one TMA box, 8 KiB
+constexpr int kDwTile = 2 * kDwHalf;
+constexpr int kDwStageBytes = 6 * kDwTile;
+
+__global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_constant__ FfTcMaps maps, FfTcDwArgs a) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    __shared__ __align__(8) uint64_t full[kDwSt], empty[kDwSt], accbar;
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t sbase = smem_addr(smem);
+    constexpr unsigned ncols = 512;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kDwSt; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&full[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&empty[s])));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&accbar)));
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        s_abort = 0;
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
+                     :: "r"(smem_addr(&s_tmem)), "r"(ncols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = s_tmem;
+    constexpr uint32_t idesc = idesc_bf16_f32_mn(kT, kT);
+    unsigned g_prod = 0, g_mma = 0, items_done = 0;
+    bool ready = false;                            // the next stage's operands are known to be there
+    const int items = a.tiles_m * a.tiles_n * a.ksplit;
+
+    for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+        const int ks = item % a.ksplit, tile = item / a.ksplit;
+        const int tm = tile % a.tiles_m, tn = tile / a.tiles_m;
+        const int kb0 = (int)((long long)a.kblocks * ks / a.ksplit);
+        const int kb1 = (int)((long long)a.kblocks * (ks + 1) / a.ksplit);
+        if (warp == 0 && lane == 0) {
+            for (int kb = kb0; kb < kb1; ++kb, ++g_prod) {
+                const int st = g_prod % kDwSt;
+                const unsigned round = g_prod / kDwSt;
+                if (round > 0 && !mbar_wait(smem_addr(&empty[st]), (round - 1) & 1u, a.ctl)) { s_abort = 1; break; }
+                const uint32_t fb = smem_addr(&full[st]);
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+                             :: "r"(fb), "r"(kDwStageBytes) : "memory");
+                const uint32_t d0 = sbase + st * kDwStageBytes;
+                // gradient parts, then the spikes 1 .. 4 steps earlier (rows
+                // before the first and past the last are zeros)
+                for (int q = 0; q < 2; ++q)
+                    for (int h = 0; h < 2; ++h)
+                        tma_load_2d(d0 + q * kDwTile + h * kDwHalf, &maps.m[1 + q], tn * kT + h * 64, kb * kKB, fb);
+                for (int d = 1; d <= 4; ++d)
+                    for (int h = 0; h < 2; ++h)
+                        tma_load_2d(d0 + (1 + d) * kDwTile + h * kDwHalf, &maps.m[0], tm * kT + h * 64,
+                                    kb * kKB - d * a.B, fb);
+            }
+        } else if (warp == 1) {
+            for (int kb = kb0; kb < kb1; ++kb, ++g_mma) {
+                const int st = g_mma % kDwSt;
+                if (!ready && !mbar_wait(smem_addr(&full[st]), (g_mma / kDwSt) & 1u, a.ctl)) { s_abort = 1; break; }
+                ready = mbar_test(smem_addr(&full[(g_mma + 1) % kDwSt]), ((g_mma + 1) / kDwSt) & 1u);
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t d0 = sbase + st * kDwStageBytes;
+#pragma unroll
+                for (int d = 0; d < 4; ++d)
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+#pragma unroll
+                        for (int kk = 0; kk < kKB / 16; ++kk)
+                            mma_bf16(tmem + d * kT, umma_desc_mn_sw128(d0 + (2 + d) * kDwTile + kk * 2048, kDwHalf),
+                                     umma_desc_mn_sw128(d0 + q * kDwTile + kk * 2048, kDwHalf), idesc,
+                                     (kb > kb0) | (q > 0) | (kk > 0));
+                mma_commit(smem_addr(&empty[st]));
+            }
+            mma_commit(smem_addr(&accbar));
+        }
+        __syncwarp();
+        const bool ok = mbar_wait(smem_addr(&accbar), items_done & 1u, a.ctl);
+        ++items_done;
+        if (!ok) s_abort = 1;
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        // epilogue as in ff_tc_kernel, each element from its own delay's accumulator
+        float *Cs = (float *)smem;                  // [128][kCPitch]
+        const int quarter = warp & 3, half = warp >> 2;
+        const int ml = quarter * 32 + lane, m = tm * kT + ml;
+        for (int cc = 0; cc < 2; ++cc) {
+            const int c0 = half * 64 + cc * 32;
+            const int n0 = tn * kT + c0;
+            float out[32];
+#pragma unroll
+            for (int q = 0; q < 32; ++q) out[q] = 0.0f;
+            for (int d = 0; d < 4; ++d) {
+                uint32_t v[32];
+                tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(d * kT + c0), v);
+                if (!ok || kb1 == kb0 || m >= a.M) continue;
+                const uint8_t *Dr = a.D + (size_t)m * a.N;
+#pragma unroll
+                for (int q = 0; q < 32; ++q)
+                    if (n0 + q < a.N && Dr[n0 + q] == d + 1) out[q] = __uint_as_float(v[q]);
+            }
+            float4 *dst = (float4 *)(Cs + ml * kCPitch + c0);
+#pragma unroll
+            for (int q4 = 0; q4 < 8; ++q4)
+                dst[q4] = make_float4(out[4 * q4], out[4 * q4 + 1], out[4 * q4 + 2], out[4 * q4 + 3]);
+        }
+        __syncthreads();
+        if (ok) {
+            float *C = a.C + (size_t)ks * a.cstride;
+            const int ncol = min(kT, a.N - tn * kT);
+            for (int row = warp; row < kT; row += kThreads / 32) {
+                const int mm = tm * kT + row;
+                if (mm >= a.M) break;
+                float *crow = C + (size_t)mm * a.N + tn * kT;
+                const float *srow = Cs + row * kCPitch;
+                for (int c = lane; c < ncol; c += 32) crow[c] = srow[c];
+            }
+        }
+        // the staged tile was written and read through the generic proxy; the
+        // next item's TMA (async proxy) reuses those bytes
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        __syncthreads();
+    }
+
+    // drain: as in ff_tc_kernel
+    if (warp == 0 && lane == 0) {
+        for (unsigned i = g_prod > kDwSt ? g_prod - kDwSt : 0; i < g_prod; ++i)
+            mbar_wait(smem_addr(&full[i % kDwSt]), (i / kDwSt) & 1u, a.ctl);
+    }
+    if (warp == 1 && lane == 0) {
+        for (unsigned i = g_mma > kDwSt ? g_mma - kDwSt : 0; i < g_mma; ++i)
+            mbar_wait(smem_addr(&empty[i % kDwSt]), (i / kDwSt) & 1u, a.ctl);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -439,63 +569,16 @@ __global__ void __launch_bounds__(256) ff_tc_weights_kernel(const float *__restr
     }
 }
 
-// Spike bits [rows][words] -> 0/1 BF16: rows S [rows][nin_p] and/or the
-// transpose ST [n_in][rows_p], whichever is given (padding stays zero).  A
-// block converts a 32 x 32 tile (rows r0.., inputs i0..) through shared
-// memory, so both outputs leave as 64-byte row pieces.
+// Spike bits [rows][words] -> 0/1 BF16 rows S [rows][nin_p] (padding stays zero).
 __global__ void __launch_bounds__(256) ff_tc_spikes_kernel(const unsigned *__restrict__ bits, int rows, int n_in,
-                                                           int words, int nin_p, int rows_p, __nv_bfloat16 *S,
-                                                           __nv_bfloat16 *ST) {
-    __shared__ __nv_bfloat16 tile[32][34];
-    const int r0 = blockIdx.x * 32, i0 = blockIdx.y * 32;   // rows on x: no 65535 limit
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // 32 x 8
+                                                           int words, int nin_p, __nv_bfloat16 *S) {
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (r >= rows) return;
     const __nv_bfloat16 one = __float2bfloat16_rn(1.0f), zero = __float2bfloat16_rn(0.0f);
-    for (int y = ty; y < 32; y += 8) {
-        const int r = r0 + y, i = i0 + tx;
-        bool sp = false;
-        if (r < rows && i < n_in) sp = (__ldg(bits + (size_t)r * words + (i >> 5)) >> (i & 31)) & 1u;
-        tile[y][tx] = sp ? one : zero;
-        if (S && r < rows && i < n_in) S[(size_t)r * nin_p + i] = sp ? one : zero;
-    }
-    if (!ST) return;
-    __syncthreads();
-    for (int y = ty; y < 32; y += 8) {
-        const int i = i0 + y, r = r0 + tx;
-        if (i < n_in && r < rows) ST[(size_t)i * rows_p + r] = tile[tx][y];
-    }
-}
-
-// Gradient gI [rows][n_out] -> two-term BF16 split G[s] ([rows][nout_p]) and,
-// if GT is given, its transpose GT[s] ([n_out][rows_p]); 32 x 32 tiles
-// through shared memory.
-__global__ void __launch_bounds__(256) ff_tc_gsplit_kernel(const float *__restrict__ g, int rows, int n_out,
-                                                           int nout_p, int rows_p, __nv_bfloat16 *G,
-                                                           __nv_bfloat16 *GT) {
-    __shared__ __nv_bfloat16 th[32][34], tm[32][34];
-    const int r0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const size_t gsz = (size_t)rows * nout_p, tsz = (size_t)n_out * rows_p;
-    for (int y = ty; y < 32; y += 8) {
-        const int r = r0 + y, j = j0 + tx;
-        float x = 0.0f;
-        if (r < rows && j < n_out) x = __ldg(g + (size_t)r * n_out + j);
-        const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-        const __nv_bfloat16 mid = __float2bfloat16_rn(__fsub_rn(x, __bfloat162float(hi)));
-        th[y][tx] = hi;
-        tm[y][tx] = mid;
-        if (G && r < rows && j < n_out) {
-            G[(size_t)r * nout_p + j] = hi;
-            G[gsz + (size_t)r * nout_p + j] = mid;
-        }
-    }
-    if (!GT) return;
-    __syncthreads();
-    for (int y = ty; y < 32; y += 8) {
-        const int j = j0 + y, r = r0 + tx;
-        if (j < n_out && r < rows) {
-            GT[(size_t)j * rows_p + r] = th[tx][y];
-            GT[tsz + (size_t)j * rows_p + r] = tm[tx][y];
-        }
+    for (int w = 0; w < words; ++w) {
+        const unsigned b = __ldg(bits + (size_t)r * words + w);
+        const int i = w * 32 + lane;
+        if (i < n_in) S[(size_t)r * nin_p + i] = (b >> lane) & 1u ? one : zero;
     }
 }
 
@@ -522,9 +605,24 @@ cudaError_t ff_tc_gemm(const FfTcMaps &maps, const FfTcArgs &args, cudaStream_t 
     if ((e = cudaFuncSetAttribute((const void *)ff_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem)) != cudaSuccess)
         return e;
-    const int items = args.tiles_m * args.tiles_n * args.ksplit;
+    const int items = args.tiles_m * args.tiles_n;
     const int grid = items < sms ? items : sms;
     ff_tc_kernel<<<grid, kThreads, smem, s>>>(maps, args);
+    return cudaGetLastError();
+}
+
+cudaError_t ff_tc_dw(const FfTcMaps &maps, const FfTcDwArgs &args, cudaStream_t s) {
+    static_assert(kT * kCPitch * 4 <= kDwSt * kDwStageBytes, "staged output tile fits the stage buffers");
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    const size_t smem = (size_t)kDwSt * kDwStageBytes + 1024;
+    if ((e = cudaFuncSetAttribute((const void *)ff_tc_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)smem)) != cudaSuccess)
+        return e;
+    const int items = args.tiles_m * args.tiles_n * args.ksplit;
+    ff_tc_dw_kernel<<<items < sms ? items : sms, kThreads, smem, s>>>(maps, args);
     return cudaGetLastError();
 }
 
@@ -552,20 +650,8 @@ cudaError_t ff_tc_weights(const float *W, const uint8_t *D, int n_in, int n_out,
     return cudaGetLastError();
 }
 
-cudaError_t ff_tc_spikes(const unsigned *bits, int rows, int n_in, int words, int nin_p, int rows_p, void *S,
-                         void *ST, cudaStream_t s) {
-    // one block per tile: a grid-stride loop over tiles measured slower
-    const dim3 grid((rows + 31) / 32, (n_in + 31) / 32);
-    ff_tc_spikes_kernel<<<grid, 256, 0, s>>>(bits, rows, n_in, words, nin_p, rows_p, (__nv_bfloat16 *)S,
-                                            (__nv_bfloat16 *)ST);
-    return cudaGetLastError();
-}
-
-cudaError_t ff_tc_gsplit(const float *g, int rows, int n_out, int nout_p, int rows_p, void *G, void *GT,
-                         cudaStream_t s) {
-    const dim3 grid((rows + 31) / 32, (n_out + 31) / 32);
-    ff_tc_gsplit_kernel<<<grid, 256, 0, s>>>(g, rows, n_out, nout_p, rows_p, (__nv_bfloat16 *)G,
-                                            (__nv_bfloat16 *)GT);
+cudaError_t ff_tc_spikes(const unsigned *bits, int rows, int n_in, int words, int nin_p, void *S, cudaStream_t s) {
+    ff_tc_spikes_kernel<<<(rows + 7) / 8, 256, 0, s>>>(bits, rows, n_in, words, nin_p, (__nv_bfloat16 *)S);
     return cudaGetLastError();
 }
 

@@ -170,9 +170,10 @@ cudaError_t ff_delay_fwd(const unsigned *sprev, int words_in, const float *W, co
 cudaError_t ff_scan_fwd(const float *I, int n, int B, int T, int k, float theta, float leak, float reset,
                         int refractory, unsigned *S, float *vck, int *rck, float *counts, void *sbf, int ldbf,
                         cudaStream_t s);
+// gI as floats [T*B][n], or (gbf given) as its two BF16 parts [2][T*B][ldg]
 cudaError_t ff_scan_bwd(const float *I, int n, int B, int T, int k, float theta, float leak, float reset,
                         int refractory, float slope, const float *vck, const int *rck, const float *gs,
-                        const float *gc, float *gI, cudaStream_t s);
+                        const float *gc, float *gI, void *gbf, int ldg, cudaStream_t s);
 cudaError_t ff_bwd_data(const float *gI, const float *W, const uint8_t *D, int n_in, int n_out, int B, int T,
                         float *gsp, cudaStream_t s);
 cudaError_t ff_dw(const float *gI, const unsigned *sprev, int words_in, const uint8_t *D, int n_in, int n_out,
@@ -182,36 +183,39 @@ cudaError_t ff_dw(const float *gI, const unsigned *sprev, int words_in, const ui
 // is a K loop over `kblocks` 64-element blocks: A tile rows a_y + 128 * tm,
 // K a_x + 64 * kb of map amap; B tile rows b_y + 128 * tn, K b_x + 64 * kb of
 // map bmap (and, with nb = 2, a second B tile from bmap2 at rows b_y2 + 128 *
-// tn, multiplying the same A tile); into accumulator acc.  mode 0: C[m][n] = acc 0; mode 1: C[m][n] =
-// acc (D[m][n] - 1) (delay-selected weight gradient).  With ksplit > 1 the
-// work item of split ks covers its share of every pass's K blocks and writes
-// C + ks * cstride.
+// tn, multiplying the same A tile); C[m][n] = the sum of all passes.
 constexpr int kFfTcMaxMaps = 4;
 constexpr int kFfTcMaxPasses = 16;
 struct FfTcMaps {
     CUtensorMap m[kFfTcMaxMaps];
 };
 struct FfTcPass {
-    int amap, bmap, a_y, a_x, b_y, b_x, kblocks, acc;
+    int amap, bmap, a_y, a_x, b_y, b_x, kblocks;
     int nb, bmap2, b_y2;              // B tiles per stage (1, or 2: the second from bmap2 at rows b_y2)
 };
 struct FfTcArgs {
-    int M, N, tiles_m, tiles_n, ksplit, npass, nacc, mode;
+    int M, N, tiles_m, tiles_n, npass;
     int part_stride;                  // forward kernel: rows between the B parts of a pass
     FfTcPass pass[kFfTcMaxPasses];
     float *C;
-    long long ldc, cstride;
-    const uint8_t *D;
+    long long ldc;
     Control *ctl;
 };
 cudaError_t ff_tc_gemm(const FfTcMaps &maps, const FfTcArgs &args, cudaStream_t s);
 cudaError_t ff_tc_forward(const FfTcMaps &maps, const FfTcArgs &args, cudaStream_t s);
 cudaError_t ff_tc_weights(const float *W, const uint8_t *D, int n_in, int n_out, int nout_p, int rows_in,
                           void *Wb, int nin_p, int rows_out, void *Wf, cudaStream_t s);
-cudaError_t ff_tc_spikes(const unsigned *bits, int rows, int n_in, int words, int nin_p, int rows_p, void *S,
-                         void *ST, cudaStream_t s);
-cudaError_t ff_tc_gsplit(const float *g, int rows, int n_out, int nout_p, int rows_p, void *G, void *GT,
-                         cudaStream_t s);
+cudaError_t ff_tc_spikes(const unsigned *bits, int rows, int n_in, int words, int nin_p, void *S, cudaStream_t s);
+// Weight gradient (ff_tc_dw_kernel): maps m[0] the spikes, m[1] and m[2] the
+// gradient's parts, boxes of 64 rows x 64 columns; C [ksplit][M][N].
+struct FfTcDwArgs {
+    int M, N, tiles_m, tiles_n, ksplit, kblocks, B;
+    float *C;
+    long long cstride;
+    const uint8_t *D;
+    Control *ctl;
+};
+cudaError_t ff_tc_dw(const FfTcMaps &maps, const FfTcDwArgs &args, cudaStream_t s);
 cudaError_t ff_dw_reduce(const float *part, int splits, long long count, float *dW, cudaStream_t s);
 
 // Launchers (kernels live in sn_kernels.cu).  Return a CUDA error code.

@@ -74,6 +74,20 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t addr) {
     return d;
 }
 
+// The same swizzle for an MN-major tile of 16-bit elements (the operand's rows
+// or columns contiguous, K in steps of 128 bytes): atoms of 64 MN elements x 8 K
+// rows (1024 bytes) follow one another along K, the next 64 MN elements lie
+// mn_stride bytes away.  A K step of 16 advances the address by 2048 bytes.
+__device__ __forceinline__ uint64_t umma_desc_mn_sw128(uint32_t addr, uint32_t mn_stride) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFFu);
+    d |= (uint64_t)(mn_stride >> 4) << 16;
+    d |= (uint64_t)(1024u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
 // Instruction descriptor of kind::f8f6f4: FP32 accumulator, A and B E4M3,
 // both K-major, N = 128, M = 128.
 __host__ __device__ constexpr uint32_t idesc_e4m3_f32(int m, int n) {
@@ -211,6 +225,11 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+
+// The same with both operands MN-major.
+__host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int m, int n) {
+    return idesc_bf16_f32(m, n) | (1u << 15) | (1u << 16);
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, int acc) {
