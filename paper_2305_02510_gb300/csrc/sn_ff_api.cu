@@ -39,34 +39,25 @@ sn_status bf16_map(sn_ctx *c, CUtensorMap *out, const void *base, long long rows
 bool use_tc(const sn_ctx *c) { return c->ff_tc_ok && c->ff_engine != SN_FF_SIMT; }
 
 // Synaptic input of layer l for all rows, I[r][j] = sum_d sum_i S[r - dB][i] W_d[i][j]:
-// 4 delays x 3 exact BF16 weight parts (4 passes of 3 parts each), accumulated
-// block by block (ff_tc_forward), from the spike operand of layer l - 1.
+// 4 delays x 3 exact BF16 weight parts, accumulated block by block (ff_tc_rows),
+// from the spike operand of layer l - 1.
 sn_status tc_forward(sn_ctx *c, int l, float *I) {
     const int B = c->ff_batch, rows = B * c->ff_steps;
     const int nin = c->ff_sizes[l - 1], nout = c->ff_sizes[l];
     const int nin_p = up(nin, 64), rows_out = up(nout, 128);
-    cudaError_t e;
     FfTcMaps maps;
     FfTcArgs a;
     memset(&maps, 0, sizeof(maps));
     memset(&a, 0, sizeof(a));
     sn_status s;
+    a.bn = nout < 128 ? up(nout, 16) : 128;
     if ((s = bf16_map(c, &maps.m[0], c->ff_Sbf[l - 1], rows, nin_p)) ||
-        (s = bf16_map(c, &maps.m[1], c->ff_Wf[l - 1], 12LL * rows_out, nin_p)))
+        (s = bf16_map(c, &maps.m[2], c->ff_Wf[l - 1], 12LL * rows_out, nin_p, a.bn)))
         return s;
-    // one pass per delay; the kernel multiplies its spike tile by the three
-    // weight parts, rows_out apart in the map
-    for (int d = 1; d <= 4; ++d) {
-        FfTcPass &ps = a.pass[a.npass++];
-        ps.amap = 0; ps.a_y = -d * B; ps.a_x = 0;
-        ps.bmap = 1; ps.b_y = (d - 1) * 3 * rows_out; ps.b_x = 0;
-        ps.kblocks = nin_p / 64;
-    }
-    a.part_stride = rows_out;
-    a.M = rows; a.N = nout;
-    a.tiles_m = (rows + 127) / 128; a.tiles_n = (nout + 127) / 128;
+    a.M = rows; a.N = nout; a.kblocks = nin_p / 64; a.shift = -B; a.part_rows = rows_out;
     a.C = I; a.ldc = nout; a.ctl = c->ctl;
-    if ((e = ff_tc_forward(maps, a, c->stream)) != cudaSuccess) return cuda_fail(c, e, "tensor-core synaptic input");
+    cudaError_t e = ff_tc_rows(maps, a, false, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core synaptic input");
     return SN_OK;
 }
 
@@ -113,7 +104,7 @@ sn_status tc_weight_grad(sn_ctx *c, int l, float *dW) {
 }
 
 // Gradient of the spikes of layer l-1: gS[r][i] = sum_d sum_j gI[r + dB][j] W_d[i][j],
-// with the two-part splits hi*hi + hi*mid + mid*hi: 12 passes.
+// with the two-part splits hi*hi + hi*mid + mid*hi.
 sn_status tc_spike_grad(sn_ctx *c, int l) {
     const int B = c->ff_batch, rows = B * c->ff_steps;
     const int nin = c->ff_sizes[l - 1], nout = c->ff_sizes[l];
@@ -124,27 +115,14 @@ sn_status tc_spike_grad(sn_ctx *c, int l) {
     memset(&a, 0, sizeof(a));
     sn_status s;
     const __nv_bfloat16 *G = (const __nv_bfloat16 *)c->ff_G;
+    a.bn = nin < 128 ? up(nin, 16) : 128;
     if ((s = bf16_map(c, &maps.m[0], G, rows, nout_p)) ||
         (s = bf16_map(c, &maps.m[1], G + (size_t)rows * nout_p, rows, nout_p)) ||
-        (s = bf16_map(c, &maps.m[2], c->ff_Wb[l - 1], 8LL * rows_in, nout_p)))
+        (s = bf16_map(c, &maps.m[2], c->ff_Wb[l - 1], 8LL * rows_in, nout_p, a.bn)))
         return s;
-    // per delay: hi gradient part times both weight parts, mid part times hi
-    for (int d = 1; d <= 4; ++d) {
-        FfTcPass &ps = a.pass[a.npass++];
-        ps.amap = 0; ps.a_y = d * B; ps.a_x = 0;
-        ps.bmap = 2; ps.b_y = (d - 1) * 2 * rows_in; ps.b_x = 0;
-        ps.nb = 2; ps.bmap2 = 2; ps.b_y2 = ((d - 1) * 2 + 1) * rows_in;
-        ps.kblocks = nout_p / 64;
-        FfTcPass &pl = a.pass[a.npass++];
-        pl.amap = 1; pl.a_y = d * B; pl.a_x = 0;
-        pl.bmap = 2; pl.b_y = (d - 1) * 2 * rows_in; pl.b_x = 0;
-        pl.nb = 1;
-        pl.kblocks = nout_p / 64;
-    }
-    a.M = rows; a.N = nin;
-    a.tiles_m = (rows + 127) / 128; a.tiles_n = (nin + 127) / 128;
+    a.M = rows; a.N = nin; a.kblocks = nout_p / 64; a.shift = B; a.part_rows = rows_in;
     a.C = c->ff_gS; a.ldc = nin; a.ctl = c->ctl;
-    cudaError_t e = ff_tc_gemm(maps, a, c->stream);
+    cudaError_t e = ff_tc_rows(maps, a, true, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core spike gradient");
     return SN_OK;
 }

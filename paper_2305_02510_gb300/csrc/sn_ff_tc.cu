@@ -1,7 +1,7 @@
 // Tensor-core (tcgen05, BF16 operands, FP32 accumulation in TMEM) contractions
-// of the feedforward network: the forward synaptic input (ff_tc_fwd_kernel)
-// and the backward's spike and weight gradients (ff_tc_kernel).  sn_ff.cu has
-// the recurrences and the SIMT forms of these contractions.
+// of the feedforward network: the forward synaptic input and the backward's spike
+// gradient (ff_tc_rows_kernel) and the weight gradient (ff_tc_dw_kernel).
+// sn_ff.cu has the recurrences and the SIMT forms of these contractions.
 //
 // A delay-shifted contraction is a sum of plain GEMMs, one per delay d, with
 // the weights restricted to the synapses of delay d (W_d = W masked by
@@ -14,22 +14,14 @@
 // exact 0/1, and the cross products hi*hi + hi*mid + mid*hi are accumulated in
 // FP32 (relative error near 2^-16 per product).
 //
-// The forward synaptic input I[r][j] = sum_d sum_i S[r - dB][i] W_d[i][j] runs
-// as 4 passes (one per delay), each multiplying a 0/1 spike tile by the three
-// BF16 parts hi + mid + lo of every weight (an exact split), so every product
-// is exact.  The forward kernel accumulates one 64-input block of all passes
-// at a time in TMEM (double-buffered) and adds each block's partial sums in
-// FP32 (round to nearest) in registers of dedicated drain warps: a sequential
-// sum over input blocks, so only 48 MMA steps ever accumulate in TMEM.
+// The forward synaptic input I[r][j] = sum_d sum_i S[r - dB][i] W_d[i][j] multiplies
+// 0/1 spikes by the three BF16 parts hi + mid + lo of every weight (an exact
+// split), so every product is exact; one 64-input block of all delays at a time
+// accumulates in TMEM, and the blocks are added in FP32 (round to nearest) in
+// registers: only 48 MMA steps ever accumulate in TMEM.
 //
-// One kernel runs a list of passes, each a K loop of 64-element (128-byte)
-// blocks of an A and one or two B tensor maps at given coordinate offsets
-// (both B tiles multiply the same A tile, which is loaded once), into one of
-// up to four TMEM accumulators of a 128 x 128 output tile.  The structure is
-// that of sn_shared.cu: warp 0 lane 0 issues TMA into a 4-stage ring, warp 1
-// lane 0 issues the MMAs, then all eight warps drain the accumulators through
-// shared memory into coalesced FP32 rows.  Work items are (tile, K split)
-// pairs taken by a persistent grid; every wait is bounded.
+// Warp 0 lane 0 issues TMA into rings of shared memory, warp 1 the MMAs; work
+// items are taken by a persistent grid; every wait is bounded.
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -45,165 +37,24 @@ namespace {
 
 constexpr int kT = 128;                         // tile rows (M) and columns (N)
 constexpr int kKB = 64;                         // BF16 elements of K per stage (128 bytes)
-constexpr int kSt = 4;
 constexpr int kStageA = kT * 128;               // 16 KiB
-constexpr int kStageBytes = 3 * kStageA;        // A and up to two B tiles: 48 KiB
 constexpr int kThreads = 256;
 constexpr int kCPitch = kT + 4;                 // floats per staged output row
 
-__global__ void __launch_bounds__(kThreads, 1) ff_tc_kernel(const __grid_constant__ FfTcMaps maps, FfTcArgs a) {
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full[kSt], empty[kSt], accbar;
-    __shared__ uint32_t s_tmem;
-    __shared__ int s_abort;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t sbase = smem_addr(smem);
-    constexpr unsigned ncols = 128;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kSt; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&full[s])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&empty[s])));
-        }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&accbar)));
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        s_abort = 0;
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
-                     :: "r"(smem_addr(&s_tmem)), "r"(ncols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t tmem = s_tmem;
-    constexpr uint32_t idesc = idesc_bf16_f32(kT, kT);
-    unsigned g_prod = 0, g_mma = 0, items_done = 0;
-    bool ready = false;                            // the next stage's operands are known to be there
-    const int items = a.tiles_m * a.tiles_n;
-
-    for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
-        const int tm = item % a.tiles_m, tn = item / a.tiles_m;
-        if (warp == 0 && lane == 0) {
-            // TMA producer over every pass's K blocks
-            for (int p = 0; p < a.npass && !s_abort; ++p) {
-                const FfTcPass &ps = a.pass[p];
-                for (int kb = 0; kb < ps.kblocks; ++kb, ++g_prod) {
-                    const int st = g_prod % kSt;
-                    const unsigned round = g_prod / kSt;
-                    if (round > 0 && !mbar_wait(smem_addr(&empty[st]), (round - 1) & 1u, a.ctl)) {
-                        s_abort = 1;
-                        break;
-                    }
-                    const uint32_t fb = smem_addr(&full[st]);
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
-                                 :: "r"(fb), "r"((1 + ps.nb) * kStageA) : "memory");
-                    const uint32_t dA = sbase + st * kStageBytes;
-                    tma_load_2d(dA, &maps.m[ps.amap], ps.a_x + kb * kKB, ps.a_y + tm * kT, fb);
-                    tma_load_2d(dA + kStageA, &maps.m[ps.bmap], ps.b_x + kb * kKB, ps.b_y + tn * kT, fb);
-                    if (ps.nb > 1)
-                        tma_load_2d(dA + 2 * kStageA, &maps.m[ps.bmap2], ps.b_x + kb * kKB, ps.b_y2 + tn * kT, fb);
-                }
-            }
-        } else if (warp == 1) {
-            // MMA issuer; the item's first MMA overwrites the accumulator.  The
-            // next stage's barrier is looked at before this stage's MMAs go out.
-            int on = 0;
-            for (int p = 0; p < a.npass && !s_abort; ++p) {
-                const FfTcPass &ps = a.pass[p];
-                for (int kb = 0; kb < ps.kblocks; ++kb, ++g_mma) {
-                    const int st = g_mma % kSt;
-                    const unsigned round = g_mma / kSt;
-                    if (!ready && !mbar_wait(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
-                    ready = mbar_test(smem_addr(&full[(g_mma + 1) % kSt]), ((g_mma + 1) / kSt) & 1u);
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t dA = sbase + st * kStageBytes;
-#pragma unroll
-                    for (int kk = 0; kk < 128 / 32; ++kk)
-                        mma_bf16(tmem, umma_desc_sw128(dA + kk * 32), umma_desc_sw128(dA + kStageA + kk * 32), idesc,
-                                 on | (kk > 0));
-                    if (ps.nb > 1) {
-#pragma unroll
-                        for (int kk = 0; kk < 128 / 32; ++kk)
-                            mma_bf16(tmem, umma_desc_sw128(dA + kk * 32), umma_desc_sw128(dA + 2 * kStageA + kk * 32),
-                                     idesc, 1);
-                    }
-                    mma_commit(smem_addr(&empty[st]));
-                    on = 1;
-                }
-            }
-            mma_commit(smem_addr(&accbar));
-        }
-        __syncwarp();
-        const bool ok = mbar_wait(smem_addr(&accbar), items_done & 1u, a.ctl);
-        ++items_done;
-        if (!ok) s_abort = 1;
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        // epilogue: warps w and w+4 read TMEM lane quarter w (tile rows), each
-        // half of the columns; values go to a staged tile in the (now idle)
-        // pipeline buffers, then leave as coalesced rows
-        float *Cs = (float *)smem;                  // [128][kCPitch]
-        const int quarter = warp & 3, half = warp >> 2;
-        const int ml = quarter * 32 + lane;
-        for (int cc = 0; cc < 2; ++cc) {
-            const int c0 = half * 64 + cc * 32;
-            uint32_t v[32];
-            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
-            float4 *dst = (float4 *)(Cs + ml * kCPitch + c0);
-#pragma unroll
-            for (int q4 = 0; q4 < 8; ++q4)
-                dst[q4] = make_float4(__uint_as_float(v[4 * q4]), __uint_as_float(v[4 * q4 + 1]),
-                                      __uint_as_float(v[4 * q4 + 2]), __uint_as_float(v[4 * q4 + 3]));
-        }
-        __syncthreads();
-        if (ok) {
-            float *C = a.C;
-            const int ncol = min(kT, a.N - tn * kT);
-            for (int row = warp; row < kT; row += kThreads / 32) {
-                const int mm = tm * kT + row;
-                if (mm >= a.M) break;
-                float *crow = C + (size_t)mm * a.ldc + tn * kT;
-                const float *srow = Cs + row * kCPitch;
-                for (int c = lane; c < ncol; c += 32) crow[c] = srow[c];
-            }
-        }
-        // the staged tile was written and read through the generic proxy; the
-        // next item's TMA (async proxy) reuses those bytes
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        __syncthreads();
-    }
-
-    // drain: copies issued and MMAs committed complete before shared memory and
-    // TMEM go away (bounded waits; no-ops when the phases have completed)
-    if (warp == 0 && lane == 0) {
-        for (unsigned i = g_prod > kSt ? g_prod - kSt : 0; i < g_prod; ++i)
-            mbar_wait(smem_addr(&full[i % kSt]), (i / kSt) & 1u, a.ctl);
-    }
-    if (warp == 1 && lane == 0) {
-        for (unsigned i = g_mma > kSt ? g_mma - kSt : 0; i < g_mma; ++i)
-            mbar_wait(smem_addr(&empty[i % kSt]), (i / kSt) & 1u, a.ctl);
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(ncols));
-}
-
 // Weight gradient: dW[i][j] = sum over the rows r of S[r - dB][i] gI[r][j], d the
 // synapse's own delay.  One 128 x 128 tile per work item with four TMEM
-// accumulators, one per delay; K is the rows, 64 a stage.  A stage holds the spike
-// tile shifted by each of the four delays and both parts of the gradient tile (96
-// KiB, 32 MMAs): the gradient is read once for the four delays (48 bytes a cycle
-// into the SM at the MMAs' full rate; one delay a stage took 94, which the L2
-// does not give).  Both operands are taken as they lie, rows of K with the inputs
-// or outputs contiguous (MN-major), so nothing is transposed for them.
-// 256 threads as in ff_tc_kernel.  12,800 rows: 1024 x 1024 183 -> 152 us, 700 x 1024
-// 130 -> 116 us, and the transposes (60 us) are gone.
+// accumulators, one per delay; K is the rows, 64 a stage.  A stage holds both parts
+// of the gradient tile and the spike tile shifted by each of the four delays (96
+// KiB, 32 MMAs): the gradient is read once for the four delays (47 bytes a cycle
+// into the SM at the MMAs' full rate; one delay at a time took 94, and the L2 gives
+// about 53).  Both operands are taken as they lie, rows of K with the inputs or
+// outputs contiguous (MN-major), so nothing is transposed for them.  What bounds it
+// is shared memory: an MMA of 128 x 128 x 16 reads 8 KiB in its 64 cycles and 3 KiB
+// are written for it, 86 cycles at 128 bytes a cycle (92 measured).  Separate rings
+// for spike tiles and gradient, freed one by one, were slower (108: a barrier and a
+// commit every 8 MMAs).  256 threads: warp 0 lane 0 TMA, warp 1 MMA, all eight the
+// epilogue.  12,800 rows: 1024 x 1024 183 -> 152 us, 700 x 1024 130 -> 116 us, and the
+// transposes (60 us) are gone.
 constexpr int kDwSt = 2;
 constexpr int kDwHalf = 64 * 128;               // 64 rows x 64 columns: one TMA box, 8 KiB
 constexpr int kDwTile = 2 * kDwHalf;
@@ -273,16 +124,12 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
                 if (!ready && !mbar_wait(smem_addr(&full[st]), (g_mma / kDwSt) & 1u, a.ctl)) { s_abort = 1; break; }
                 ready = mbar_test(smem_addr(&full[(g_mma + 1) % kDwSt]), ((g_mma + 1) / kDwSt) & 1u);
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t d0 = sbase + st * kDwStageBytes;
+                const uint64_t d0 = umma_desc_mn_sw128(sbase + st * kDwStageBytes, kDwHalf);
 #pragma unroll
-                for (int d = 0; d < 4; ++d)
-#pragma unroll
-                    for (int q = 0; q < 2; ++q)
-#pragma unroll
-                        for (int kk = 0; kk < kKB / 16; ++kk)
-                            mma_bf16(tmem + d * kT, umma_desc_mn_sw128(d0 + (2 + d) * kDwTile + kk * 2048, kDwHalf),
-                                     umma_desc_mn_sw128(d0 + q * kDwTile + kk * 2048, kDwHalf), idesc,
-                                     (kb > kb0) | (q > 0) | (kk > 0));
+                for (int d = 0; d < 4; ++d) {
+                    mma_bf16_x4<128>(tmem + d * kT, d0 + (2 + d) * (kDwTile / 16), d0, idesc, kb > kb0);
+                    mma_bf16_x4<128>(tmem + d * kT, d0 + (2 + d) * (kDwTile / 16), d0 + kDwTile / 16, idesc, 1);
+                }
                 mma_commit(smem_addr(&empty[st]));
             }
             mma_commit(smem_addr(&accbar));
@@ -293,7 +140,9 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
         if (!ok) s_abort = 1;
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        // epilogue as in ff_tc_kernel, each element from its own delay's accumulator
+        // epilogue: warps w and w + 4 read TMEM lane quarter w (tile rows), each
+        // half of the columns, every element from its own delay's accumulator;
+        // the values leave as coalesced rows through the (now idle) stages
         float *Cs = (float *)smem;                  // [128][kCPitch]
         const int quarter = warp & 3, half = warp >> 2;
         const int ml = quarter * 32 + lane, m = tm * kT + ml;
@@ -336,7 +185,8 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
         __syncthreads();
     }
 
-    // drain: as in ff_tc_kernel
+    // drain: copies issued and MMAs committed complete before shared memory and
+    // TMEM go away (bounded waits; no-ops when the phases have completed)
     if (warp == 0 && lane == 0) {
         for (unsigned i = g_prod > kDwSt ? g_prod - kDwSt : 0; i < g_prod; ++i)
             mbar_wait(smem_addr(&full[i % kDwSt]), (i / kDwSt) & 1u, a.ctl);
@@ -351,41 +201,57 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(ncols));
 }
 
-// Forward synaptic input with block-wise accumulation.  384 threads: warp 0
-// lane 0 issues TMA (K block outer, pass inner), warp 1 lane 0 issues the
-// MMAs of one K block of every pass into TMEM buffer (block & 1) and commits
-// it to accf[buf]; warps 4..11 (warp w: TMEM lane quarter w % 4, columns
-// 64 * ((w - 4) / 4) ..+63) add each block's partial into FP32 registers and
-// release the buffer through acce[buf] (8 arrivals).  Every pass has the
-// same number of K blocks; a.C[m][n] = the sum (mode 0 layout).  A pass
-// multiplies its A tile by kFwdParts B tiles (rows b_y + s * a.part_stride,
-// s = 0 .. kFwdParts-1: the parts of one weight split), so a stage holds one
-// A tile and kFwdParts B tiles and A is read once for all parts.
-constexpr int kFwdTcThreads = 384;
-constexpr int kFwdParts = 3;
-constexpr int kFwdStageBytes = (1 + kFwdParts) * kStageA;   // 64 KiB
-constexpr int kFwdSt = 3;
+// Forward synaptic input and spike gradient: C[r][n] = sum over the delays d, the
+// K blocks kb and the products (A part, B part) of A[r + shift d][kb] B_d[n][kb].
+//   forward (SG = false): A the spikes, shift -B, three B parts (hi, mid, lo);
+//   spike gradient (SG): A parts hi, mid of the gradient, shift +B, B parts hi,
+//   mid; products hi hi, hi mid, mid hi.
+// A work item is H tiles of 128 rows x one tile of 128 columns.  Two row tiles share
+// each weight tile: with one, the operands come in at 85 bytes a cycle at the MMAs'
+// full rate, with two at 52 (forward) and 62 (the L2 gives an SM about 53).  What
+// then bounds it is shared memory: 8 KiB read by an MMA in its 64 cycles and 3.4 (4)
+// KiB written for it, 89 (94) cycles at 128 bytes a cycle; 92 and 94 measured.  The
+// operands go through two rings, units of one A part (H tiles) and of one B part, so
+// that each is freed as soon as its last MMA is done; the weights run one (kb, d)
+// step ahead of the rows.
+// A chunk of steps accumulates in TMEM (two buffers), and the drain warps add it
+// into FP32 registers: the forward's chunk is one K block (all delays: 48 MMA steps
+// in TMEM at most, a sequential sum over K blocks in round to nearest), the spike
+// gradient's the whole item.  384 threads: warp 0 lane 0 TMA, warp 1 MMA, warps 4..11
+// drain (warp w: TMEM lane quarter w % 4, columns 64 * ((w - 4) / 4) ..+63).
+// A layer of at most 112 columns loads and multiplies only those (bn).
+// 12,800 rows, forward: 1024 x 1024 228 -> 202 us, 700 x 1024 161 -> 145; spike
+// gradient: 1024 x 1024 282 -> 209, 1024 x 20 52 -> 33.
+constexpr int kRowsThreads = 384;
 
-__global__ void __launch_bounds__(kFwdTcThreads, 1) ff_tc_fwd_kernel(const __grid_constant__ FfTcMaps maps,
-                                                                     FfTcArgs a) {
+template <int H, bool SG>
+struct Rows {
+    static constexpr int NA = SG ? 2 : 1, NB = SG ? 2 : 3;        // parts of a step
+    static constexpr int RA = SG ? 4 : H == 2 ? 2 : 4;            // units in the rings
+    static constexpr int RB = H == 2 ? (SG ? 5 : 9) : (SG ? 8 : 9);
+    static constexpr int kUnitA = H * kStageA;
+    static constexpr int kBytes = RA * kUnitA + RB * kStageA;
+};
+
+template <int H, bool SG>
+__global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __grid_constant__ FfTcMaps maps, FfTcArgs a) {
+    using R = Rows<H, SG>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full[kFwdSt], empty[kFwdSt], accf[2], acce[2];
+    __shared__ __align__(8) uint64_t fullA[R::RA], emptyA[R::RA], fullB[R::RB], emptyB[R::RB], accf[2], acce[2];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t sbase = smem_addr(smem);
-    constexpr unsigned ncols = 256;
+    const uint32_t baseA = smem_addr(smem), baseB = baseA + R::RA * R::kUnitA;
+    constexpr unsigned ncols = 2 * H * kT;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kFwdSt; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&full[s])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&empty[s])));
-        }
-        for (int b = 0; b < 2; ++b) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_addr(&accf[b])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;\n" :: "r"(smem_addr(&acce[b])));
-        }
+        auto init = [](uint64_t *b, int n) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" :: "r"(smem_addr(b)), "r"(n));
+        };
+        for (int q = 0; q < R::RA; ++q) { init(&fullA[q], 1); init(&emptyA[q], 1); }
+        for (int q = 0; q < R::RB; ++q) { init(&fullB[q], 1); init(&emptyB[q], 1); }
+        for (int q = 0; q < 2; ++q) { init(&accf[q], 1); init(&acce[q], 8); }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         s_abort = 0;
@@ -399,59 +265,114 @@ __global__ void __launch_bounds__(kFwdTcThreads, 1) ff_tc_fwd_kernel(const __gri
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = s_tmem;
-    constexpr uint32_t idesc = idesc_bf16_f32(kT, kT);
-    const int items = a.tiles_m * a.tiles_n;
-    const int KB = a.pass[0].kblocks;
-    unsigned g_prod = 0, g_mma = 0;
+    const int items = a.tiles_m * a.tiles_n, steps = 4 * a.kblocks;   // step s: K block s / 4, delay s % 4 + 1
+    const int chunk = SG ? steps : 4, chunks = steps / chunk;
+    unsigned ua = 0, ub = 0;                       // units this thread has put through (or taken from) the rings
 
     if (warp == 0 && lane == 0) {
+        const int bytesB = a.bn * 128;
         for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
             const int tm = item % a.tiles_m, tn = item / a.tiles_m;
-            for (int kb = 0; kb < KB && !s_abort; ++kb)
-                for (int p = 0; p < a.npass; ++p, ++g_prod) {
-                    const FfTcPass &ps = a.pass[p];
-                    const int st = g_prod % kFwdSt;
-                    const unsigned round = g_prod / kFwdSt;
-                    if (round > 0 && !mbar_wait(smem_addr(&empty[st]), (round - 1) & 1u, a.ctl)) {
-                        s_abort = 1;
-                        break;
-                    }
-                    const uint32_t fb = smem_addr(&full[st]);
+            auto loadA = [&](int s) {
+                const int y = tm * H * kT + a.shift * (s % 4 + 1), x = s / 4 * kKB;
+                for (int p = 0; p < R::NA; ++p, ++ua) {
+                    const unsigned st = ua % R::RA, round = ua / R::RA;
+                    if (round > 0 && !mbar_wait(smem_addr(&emptyA[st]), (round - 1) & 1u, a.ctl)) { s_abort = 1; return; }
+                    const uint32_t fb = smem_addr(&fullA[st]);
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
-                                 :: "r"(fb), "r"(kFwdStageBytes) : "memory");
-                    const uint32_t dA = sbase + st * kFwdStageBytes;
-                    tma_load_2d(dA, &maps.m[ps.amap], ps.a_x + kb * kKB, ps.a_y + tm * kT, fb);
-#pragma unroll
-                    for (int q = 0; q < kFwdParts; ++q)
-                        tma_load_2d(dA + (1 + q) * kStageA, &maps.m[ps.bmap], ps.b_x + kb * kKB,
-                                    ps.b_y + q * a.part_stride + tn * kT, fb);
+                                 :: "r"(fb), "r"(R::kUnitA) : "memory");
+                    for (int h = 0; h < H; ++h)
+                        tma_load_2d(baseA + st * R::kUnitA + h * kStageA, &maps.m[p], x, y + h * kT, fb);
                 }
+            };
+            auto loadB = [&](int s) {
+                const int x = s / 4 * kKB;
+                for (int p = 0; p < R::NB; ++p, ++ub) {
+                    const unsigned st = ub % R::RB, round = ub / R::RB;
+                    if (round > 0 && !mbar_wait(smem_addr(&emptyB[st]), (round - 1) & 1u, a.ctl)) { s_abort = 1; return; }
+                    const uint32_t fb = smem_addr(&fullB[st]);
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+                                 :: "r"(fb), "r"(bytesB) : "memory");
+                    tma_load_2d(baseB + st * kStageA, &maps.m[2], x, (s % 4 * R::NB + p) * a.part_rows + tn * kT, fb);
+                }
+            };
+            loadB(0);
+            for (int s = 0; s < steps && !s_abort; ++s) {
+                loadA(s);
+                if (s + 1 < steps && !s_abort) loadB(s + 1);
+            }
         }
     } else if (warp == 1) {
-        bool ready = false;                        // the next stage's operands are known to be there
+        const uint32_t idesc = idesc_bf16_f32(kT, a.bn);
+        const uint64_t descA = umma_desc_sw128(baseA), descB = umma_desc_sw128(baseB);
         unsigned g_chunk = 0;
+        // barriers are looked at before the MMAs in front of theirs go out
+        bool seenA = false, seenB = false;
+        auto waitA = [&](unsigned u) {
+            const bool ok = seenA || mbar_wait(smem_addr(&fullA[u % R::RA]), (u / R::RA) & 1u, a.ctl);
+            seenA = false;
+            return ok;
+        };
+        auto waitB = [&](unsigned u) {
+            const bool ok = seenB || mbar_wait(smem_addr(&fullB[u % R::RB]), (u / R::RB) & 1u, a.ctl);
+            seenB = false;
+            return ok;
+        };
+        auto lookA = [&](unsigned u) { seenA = mbar_test(smem_addr(&fullA[u % R::RA]), (u / R::RA) & 1u); };
+        auto lookB = [&](unsigned u) { seenB = mbar_test(smem_addr(&fullB[u % R::RB]), (u / R::RB) & 1u); };
         for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x)
-            for (int kb = 0; kb < KB && !s_abort; ++kb, ++g_chunk) {
+            for (int c = 0; c < chunks && !s_abort; ++c, ++g_chunk) {
                 const unsigned buf = g_chunk & 1u, use = g_chunk >> 1;
                 if (use > 0 && !mbar_wait(smem_addr(&acce[buf]), (use - 1) & 1u, a.ctl)) { s_abort = 1; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t tacc = tmem + buf * kT;
-                for (int p = 0; p < a.npass; ++p, ++g_mma) {
-                    const int st = g_mma % kFwdSt;
-                    const unsigned round = g_mma / kFwdSt;
-                    if (!ready && !mbar_wait(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
-                    ready = mbar_test(smem_addr(&full[(g_mma + 1) % kFwdSt]), ((g_mma + 1) / kFwdSt) & 1u);
+                const uint32_t tacc = tmem + buf * (H * kT);
+                auto product = [&](unsigned u, unsigned v, int on) {
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t dA = sbase + st * kFwdStageBytes;
+                    const uint64_t dA = descA + u % R::RA * (R::kUnitA / 16), dB = descB + v % R::RB * (kStageA / 16);
 #pragma unroll
-                    for (int q = 0; q < kFwdParts; ++q)
-#pragma unroll
-                        for (int kk = 0; kk < 128 / 32; ++kk)
-                            mma_bf16(tacc, umma_desc_sw128(dA + kk * 32),
-                                     umma_desc_sw128(dA + (1 + q) * kStageA + kk * 32), idesc,
-                                     (p > 0) | (q > 0) | (kk > 0));
-                    mma_commit(smem_addr(&empty[st]));
+                    for (int h = 0; h < H; ++h)
+                        mma_bf16_x4<2>(tacc + h * kT, dA + h * (kStageA / 16), dB, idesc, on);
+                };
+                int s = 0;
+                for (; s < chunk; ++s) {
+                    const int on = s > 0;
+                    if constexpr (!SG) {
+                        if (!waitA(ua) || !waitB(ub)) { s_abort = 1; break; }
+                        lookB(ub + 1);
+                        product(ua, ub, on);
+                        mma_commit(smem_addr(&emptyB[ub % R::RB]));
+                        if (!waitB(ub + 1)) { s_abort = 1; break; }
+                        lookB(ub + 2);
+                        product(ua, ub + 1, 1);
+                        mma_commit(smem_addr(&emptyB[(ub + 1) % R::RB]));
+                        if (!waitB(ub + 2)) { s_abort = 1; break; }
+                        lookA(ua + 1);
+                        lookB(ub + 3);
+                        product(ua, ub + 2, 1);
+                        mma_commit(smem_addr(&emptyB[(ub + 2) % R::RB]));
+                        mma_commit(smem_addr(&emptyA[ua % R::RA]));
+                        ua += 1;
+                        ub += 3;
+                    } else {
+                        if (!waitA(ua) || !waitB(ub)) { s_abort = 1; break; }
+                        lookB(ub + 1);
+                        product(ua, ub, on);
+                        if (!waitB(ub + 1)) { s_abort = 1; break; }
+                        lookA(ua + 1);
+                        product(ua, ub + 1, 1);
+                        mma_commit(smem_addr(&emptyA[ua % R::RA]));
+                        mma_commit(smem_addr(&emptyB[(ub + 1) % R::RB]));
+                        if (!waitA(ua + 1)) { s_abort = 1; break; }
+                        lookA(ua + 2);
+                        lookB(ub + 2);
+                        product(ua + 1, ub, 1);
+                        mma_commit(smem_addr(&emptyA[(ua + 1) % R::RA]));
+                        mma_commit(smem_addr(&emptyB[ub % R::RB]));
+                        ua += 2;
+                        ub += 2;
+                    }
                 }
+                if (s < chunk) break;
                 mma_commit(smem_addr(&accf[buf]));
             }
     } else if (warp >= 4) {
@@ -459,41 +380,49 @@ __global__ void __launch_bounds__(kFwdTcThreads, 1) ff_tc_fwd_kernel(const __gri
         unsigned g_chunk = 0;
         for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
             const int tm = item % a.tiles_m, tn = item / a.tiles_m;
-            float acc[64];
+            float acc[H][64];
 #pragma unroll
-            for (int q = 0; q < 64; ++q) acc[q] = 0.0f;
+            for (int h = 0; h < H; ++h)
+#pragma unroll
+                for (int q = 0; q < 64; ++q) acc[h][q] = 0.0f;
             bool ok = true;
-            for (int kb = 0; kb < KB; ++kb, ++g_chunk) {
+            for (int c = 0; c < chunks; ++c, ++g_chunk) {
                 const unsigned buf = g_chunk & 1u, use = g_chunk >> 1;
                 ok = ok && mbar_wait(smem_addr(&accf[buf]), use & 1u, a.ctl);
                 __syncwarp();
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t v[32];
-                    tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kT + (uint32_t)(half * 64 + h * 32), v);
+                for (int h = 0; h < H; ++h)
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) acc[h * 32 + q] = __fadd_rn(acc[h * 32 + q], __uint_as_float(v[q]));
-                }
+                    for (int w = 0; w < 4; ++w) {
+                        uint32_t v[16];
+                        tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) +
+                                      (uint32_t)((buf * H + h) * kT + half * 64 + w * 16), v);
+#pragma unroll
+                        for (int q = 0; q < 16; ++q)
+                            acc[h][w * 16 + q] = __fadd_rn(acc[h][w * 16 + q], __uint_as_float(v[q]));
+                    }
                 asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" :: "r"(smem_addr(&acce[buf])) : "memory");
                 if (!ok) break;
             }
             if (!ok) { s_abort = 1; break; }
-            const int m = tm * kT + quarter * 32 + lane;
             const int n0 = tn * kT + half * 64;
-            if (m < a.M) {
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const int m = (tm * H + h) * kT + quarter * 32 + lane;
+                if (m >= a.M) continue;
                 float *crow = a.C + (size_t)m * a.ldc;
                 if (n0 + 64 <= a.N && (a.ldc & 3) == 0) {
 #pragma unroll
                     for (int q4 = 0; q4 < 16; ++q4)
                         *(float4 *)(crow + n0 + 4 * q4) =
-                            make_float4(acc[4 * q4], acc[4 * q4 + 1], acc[4 * q4 + 2], acc[4 * q4 + 3]);
+                            make_float4(acc[h][4 * q4], acc[h][4 * q4 + 1], acc[h][4 * q4 + 2], acc[h][4 * q4 + 3]);
                 } else {
 #pragma unroll
                     for (int q = 0; q < 64; ++q)
-                        if (n0 + q < a.N) crow[n0 + q] = acc[q];
+                        if (n0 + q < a.N) crow[n0 + q] = acc[h][q];
                 }
             }
         }
@@ -503,12 +432,14 @@ __global__ void __launch_bounds__(kFwdTcThreads, 1) ff_tc_fwd_kernel(const __gri
     // drain: copies issued and MMAs committed complete before shared memory and
     // TMEM go away (bounded waits; no-ops when the phases have completed)
     if (warp == 0 && lane == 0) {
-        for (unsigned i = g_prod > kFwdSt ? g_prod - kFwdSt : 0; i < g_prod; ++i)
-            mbar_wait(smem_addr(&full[i % kFwdSt]), (i / kFwdSt) & 1u, a.ctl);
+        for (unsigned i = ua > R::RA ? ua - R::RA : 0; i < ua; ++i)
+            mbar_wait(smem_addr(&fullA[i % R::RA]), (i / R::RA) & 1u, a.ctl);
+        for (unsigned i = ub > R::RB ? ub - R::RB : 0; i < ub; ++i)
+            mbar_wait(smem_addr(&fullB[i % R::RB]), (i / R::RB) & 1u, a.ctl);
     }
     if (warp == 1 && lane == 0) {
-        for (unsigned i = g_mma > kFwdSt ? g_mma - kFwdSt : 0; i < g_mma; ++i)
-            mbar_wait(smem_addr(&empty[i % kFwdSt]), (i / kFwdSt) & 1u, a.ctl);
+        for (unsigned i = ua > R::RA ? ua - R::RA : 0; i < ua; ++i)
+            mbar_wait(smem_addr(&emptyA[i % R::RA]), (i / R::RA) & 1u, a.ctl);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -591,24 +522,30 @@ static int tile_grid(long long tiles) {
 
 }  // namespace
 
-size_t ff_tc_smem_bytes() { return (size_t)kSt * kStageBytes + 1024; }
+template <int H, bool SG>
+static cudaError_t rows_launch(const FfTcMaps &maps, FfTcArgs args, int sms, cudaStream_t s) {
+    const size_t smem = (size_t)Rows<H, SG>::kBytes + 1024;
+    cudaError_t e = cudaFuncSetAttribute((const void *)ff_tc_rows_kernel<H, SG>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    args.tiles_m = (args.M + H * kT - 1) / (H * kT);
+    args.tiles_n = (args.N + kT - 1) / kT;
+    const int items = args.tiles_m * args.tiles_n;
+    ff_tc_rows_kernel<H, SG><<<items < sms ? items : sms, kRowsThreads, smem, s>>>(maps, args);
+    return cudaGetLastError();
+}
 
-cudaError_t ff_tc_gemm(const FfTcMaps &maps, const FfTcArgs &args, cudaStream_t s) {
-    static_assert(kT * kCPitch * 4 <= kSt * kStageBytes, "staged output tile fits the stage buffers");
+cudaError_t ff_tc_rows(const FfTcMaps &maps, const FfTcArgs &args, bool spike_grad, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    for (int p = 0; p < args.npass; ++p)
-        if (args.pass[p].nb < 1 || args.pass[p].nb > 2) return cudaErrorInvalidValue;
-    const size_t smem = ff_tc_smem_bytes();
-    if ((e = cudaFuncSetAttribute((const void *)ff_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem)) != cudaSuccess)
-        return e;
-    const int items = args.tiles_m * args.tiles_n;
-    const int grid = items < sms ? items : sms;
-    ff_tc_kernel<<<grid, kThreads, smem, s>>>(maps, args);
-    return cudaGetLastError();
+    // two row tiles an item once single ones fill the SMs more than once: a
+    // pair takes 1.2 to 1.3 times as long as a single one
+    const long long singles = (long long)((args.M + kT - 1) / kT) * ((args.N + kT - 1) / kT);
+    if (singles > sms)
+        return spike_grad ? rows_launch<2, true>(maps, args, sms, s) : rows_launch<2, false>(maps, args, sms, s);
+    return spike_grad ? rows_launch<1, true>(maps, args, sms, s) : rows_launch<1, false>(maps, args, sms, s);
 }
 
 cudaError_t ff_tc_dw(const FfTcMaps &maps, const FfTcDwArgs &args, cudaStream_t s) {
@@ -623,23 +560,6 @@ cudaError_t ff_tc_dw(const FfTcMaps &maps, const FfTcDwArgs &args, cudaStream_t 
         return e;
     const int items = args.tiles_m * args.tiles_n * args.ksplit;
     ff_tc_dw_kernel<<<items < sms ? items : sms, kThreads, smem, s>>>(maps, args);
-    return cudaGetLastError();
-}
-
-cudaError_t ff_tc_forward(const FfTcMaps &maps, const FfTcArgs &args, cudaStream_t s) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    for (int p = 1; p < args.npass; ++p)
-        if (args.pass[p].kblocks != args.pass[0].kblocks) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)kFwdSt * kFwdStageBytes + 1024;
-    if ((e = cudaFuncSetAttribute((const void *)ff_tc_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem)) != cudaSuccess)
-        return e;
-    const int items = args.tiles_m * args.tiles_n;
-    const int grid = items < sms ? items : sms;
-    ff_tc_fwd_kernel<<<grid, kFwdTcThreads, smem, s>>>(maps, args);
     return cudaGetLastError();
 }
 

@@ -179,30 +179,23 @@ cudaError_t ff_bwd_data(const float *gI, const float *W, const uint8_t *D, int n
 cudaError_t ff_dw(const float *gI, const unsigned *sprev, int words_in, const uint8_t *D, int n_in, int n_out,
                   int B, int T, int splits, float *part, float *dW, cudaStream_t s);
 
-// Tensor-core contractions of the feedforward network (sn_ff_tc.cu).  A pass
-// is a K loop over `kblocks` 64-element blocks: A tile rows a_y + 128 * tm,
-// K a_x + 64 * kb of map amap; B tile rows b_y + 128 * tn, K b_x + 64 * kb of
-// map bmap (and, with nb = 2, a second B tile from bmap2 at rows b_y2 + 128 *
-// tn, multiplying the same A tile); C[m][n] = the sum of all passes.
-constexpr int kFfTcMaxMaps = 4;
-constexpr int kFfTcMaxPasses = 16;
+// Tensor-core contractions of the feedforward network (sn_ff_tc.cu).
+// ff_tc_rows: C[r][n] over the delays d = 1..4, K blocks of 64 and part products.
+// Maps: m[0], m[1] the A parts (rows, boxes of 128 x 64; the forward has m[0] only),
+// m[2] the B parts (boxes of bn x 64), part p of delay d from row ((d - 1) * parts +
+// p) * part_rows.  A's rows are shifted by shift * d.  bn: columns of a tile (128, or
+// the whole of a narrower C rounded up to 16).
+constexpr int kFfTcMaxMaps = 3;
 struct FfTcMaps {
     CUtensorMap m[kFfTcMaxMaps];
 };
-struct FfTcPass {
-    int amap, bmap, a_y, a_x, b_y, b_x, kblocks;
-    int nb, bmap2, b_y2;              // B tiles per stage (1, or 2: the second from bmap2 at rows b_y2)
-};
 struct FfTcArgs {
-    int M, N, tiles_m, tiles_n, npass;
-    int part_stride;                  // forward kernel: rows between the B parts of a pass
-    FfTcPass pass[kFfTcMaxPasses];
+    int M, N, tiles_m, tiles_n, kblocks, shift, part_rows, bn;
     float *C;
     long long ldc;
     Control *ctl;
 };
-cudaError_t ff_tc_gemm(const FfTcMaps &maps, const FfTcArgs &args, cudaStream_t s);
-cudaError_t ff_tc_forward(const FfTcMaps &maps, const FfTcArgs &args, cudaStream_t s);
+cudaError_t ff_tc_rows(const FfTcMaps &maps, const FfTcArgs &args, bool spike_grad, cudaStream_t s);
 cudaError_t ff_tc_weights(const float *W, const uint8_t *D, int n_in, int n_out, int nout_p, int rows_in,
                           void *Wb, int nin_p, int rows_out, void *Wf, cudaStream_t s);
 cudaError_t ff_tc_spikes(const unsigned *bits, int rows, int n_in, int words, int nin_p, void *S, cudaStream_t s);

@@ -146,6 +146,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
+// A 16-column TMEM load and the wait for it.
+__device__ __forceinline__ void tmem_ld16(uint32_t ta, uint32_t (&a)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]),
+          "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]),
+          "=r"(a[15])
+        : "r"(ta)
+        : "memory");
+}
+
 // Two 16-column TMEM loads (this warp's lane quarter, one lane per thread)
 // and the wait for both, in one statement so that no use of the registers
 // can be scheduled before the wait.
@@ -232,11 +245,22 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int m, int n) {
     return idesc_bf16_f32(m, n) | (1u << 15) | (1u << 16);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, int acc) {
+// Four MMAs of K = 16 under one election, the descriptors advancing by STEP
+// 16-byte units (2: 32 bytes of a K-major row; 128: 16 rows of an MN-major tile).
+// Descriptors put together for each MMA took the issuing warp about 100 cycles an
+// MMA; a running sum from one descriptor costs next to nothing.
+template <int STEP>
+__device__ __forceinline__ void mma_bf16_x4(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, int acc) {
     asm volatile(
-        "{\n.reg .pred p, q;\nelect.sync _|q, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-        :: "r"(tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
+        "{\n.reg .pred p, q, t;\n.reg .b64 a1, a2, a3, b1, b2, b3;\n"
+        "elect.sync _|q, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\nsetp.eq.u32 t, 0, 0;\n"
+        "add.u64 a1, %1, %5;\nadd.u64 a2, %1, %6;\nadd.u64 a3, %1, %7;\n"
+        "add.u64 b1, %2, %5;\nadd.u64 b2, %2, %6;\nadd.u64 b3, %2, %7;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, t;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, t;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, t;\n}\n"
+        :: "r"(tmem), "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "n"(STEP), "n"(2 * STEP), "n"(3 * STEP));
 }
 
 }  // namespace sn
