@@ -706,7 +706,7 @@ sn_status sn_create_dense(const sn_config *cfg, const sn_neurons *nr, const floa
     c->S = 1;
     c->ring_bytes = (size_t)c->D1 * n * 4;
     if ((s = dalloc(c, &c->W, nn * 4)) || (s = dalloc(c, &c->spk, (size_t)2 * c->words * 4)) ||
-        (s = dalloc(c, &c->ring, c->ring_bytes)))
+        (dense_tag_bytes(n) && (s = dalloc(c, &c->ptag, dense_tag_bytes(n)))) || (s = dalloc(c, &c->ring, c->ring_bytes)))
         return bail(s);
     if ((e = w ? cudaMemcpy(c->W, w, nn * 4, cudaMemcpyHostToDevice) : cudaMemset(c->W, 0, nn * 4)) ||
         (e = cudaMemset(c->spk, 0, (size_t)2 * c->words * 4)) || (e = cudaMemset(c->ring, 0, c->ring_bytes))) {
@@ -954,8 +954,11 @@ sn_status sn_run(sn_ctx *c, int32_t steps) {
             a.chunk = c->reg_chunk;
             e = launch_sparse_reg(a, c->dtype, c->reg_grid, c->stream);
         } else {
+            a.ptag = c->ptag;
             e = c->kind == KIND_SPARSE ? launch_sparse(a, c->dtype, c->grid, c->block, c->stream)
-                                       : launch_dense(a, c->grid, c->block, c->stream);
+                : dense_res_fits(c->n, c->chunk, c->grid, c->stdp != 0, steps)
+                    ? launch_dense_res(a, c->grid, c->stream)
+                    : launch_dense(a, c->grid, c->block, c->stream);
         }
         if (e != cudaSuccess) return cuda_fail(c, e, "simulation launch");
         c->ring_live_until = c->step + steps + c->D;

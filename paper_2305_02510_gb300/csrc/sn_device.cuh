@@ -49,6 +49,13 @@ __device__ __forceinline__ int ld_status(const Control *ctl) {
     return *(volatile const int *)&ctl->status;
 }
 
+// A spike word that says itself which step it is of: the step's number in the
+// high half, stored and read as one 64-bit word.
+__device__ __forceinline__ void st_tagged(unsigned long long *p, unsigned tag, unsigned bits) {
+    const unsigned long long v = ((unsigned long long)tag << 32) | bits;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
+}
+
 // Grid-wide barrier for a cooperative launch, on a counter that only grows
 // during a launch (the host zeroes it before every launch): thread 0 of each
 // block adds one with release semantics and waits until the count reaches the

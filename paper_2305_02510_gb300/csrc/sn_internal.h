@@ -75,8 +75,8 @@ struct NetArgs {
     const unsigned *pin_y0;           // coded store: [2][n] window bit offset of each region's first entry
     const int *pin_perm;              // [n] the neuron whose lists thread position p sums (the store,
                                       // pin_len and pin_y0 are indexed by position)
-    unsigned long long *ptag;         // blocked pull: spike words of the last steps with the step's
-                                      // number in the high half (sn_pull_block.cu)
+    unsigned long long *ptag;         // blocked pull, resident dense: spike words of the last steps with
+                                      // the step's number in the high half
     int wp, wt, rows_at, acc_at;     // blocked pull: words rounded up to 4 and to 2, bytes of shared
                                       // memory before the two rows and before the sums
     unsigned *hist;                   // [hD][words] spike bits of step tau in row tau % hD
@@ -218,6 +218,12 @@ cudaError_t max_grid_sparse(int dtype, int stdp, int block, int *grid);
 cudaError_t max_grid_sparse_reg(int *grid);
 cudaError_t launch_sparse_reg(const NetArgs &a, int dtype, int grid, cudaStream_t s);
 constexpr int kSparseRegBlock = 512;
+// sn_dense_res.cu: the form that keeps W in shared memory, and its rule
+constexpr int kDenseResSteps = 4, kDenseResStepsStdp = 12;   // shortest runs that take it
+constexpr int kDenseTagStride = 16;        // 64-bit words from one spike word of a tagged row to the next
+size_t dense_tag_bytes(int n);             // 0: n never takes it
+bool dense_res_fits(int n, int chunk, int grid, bool stdp, int steps);
+cudaError_t launch_dense_res(const NetArgs &a, int grid, cudaStream_t s);
 cudaError_t plan_dense(int n, int *grid, int *chunk, int force_cpl = 0);
 // Pull propagation (sn_pull.cu).  plan_pull sets *grid = 0 when the network
 // does not fit the executor (a window of max_delay spike rows above a block's

@@ -402,7 +402,8 @@ cudaError_t max_grid_sparse(int dtype, int stdp, int block, int *grid) {
 }
 
 // ---------------------------------------------------------------------------
-// Dense network: W[n][n] row-major (row = pre), one grid barrier per step.
+// Dense network whose rows come from memory (sn_dense_res.cu runs the ones that
+// fit in shared memory): W[n][n] row-major (row = pre), one grid barrier per step.
 // Block c owns the column slab [c * cw, c * cw + cw), cw = 32 * CPL, and the
 // neurons with the same indices.  Step t:
 //   update(t):  own neurons (state in registers, parameters in shared

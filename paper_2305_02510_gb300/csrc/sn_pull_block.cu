@@ -193,10 +193,6 @@ __device__ __forceinline__ ulonglong2 ld_tagged2(const unsigned long long *p) {
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_tagged(unsigned long long *p, unsigned tag, unsigned bits) {
-    const unsigned long long v = ((unsigned long long)tag << 32) | bits;
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
-}
 
 // The tagged row of a step into shared memory, once every word carries `tag`.
 // Bounded: false when another block latched a status or the wall-clock limit
