@@ -134,9 +134,9 @@ constexpr int kBatchBlock = 256;
 constexpr int kBatchMaxN = 4096;      // largest network of a batched context
 constexpr int kBatchMaxDelay = 16;
 
-cudaError_t launch_batch(const BatchArgs &a, int dtype, int grid, cudaStream_t s);
-cudaError_t batch_kernel_node(int dtype, void **fn);
-cudaError_t max_grid_batch(int dtype, int ring_smem, int *grid);
+bool batch_own_fits(int max_block_n, int max_warp_n);
+cudaError_t batch_kernel_node(int dtype, bool own, void **fn);
+cudaError_t max_grid_batch(int dtype, bool own, int ring_smem, int *grid);
 size_t batch_smem(int ring_smem);
 
 // Shared dense network on tensor cores: sn_shared.cu, and sn_shared_res.cu when
