@@ -186,11 +186,10 @@ __device__ __forceinline__ void add_shared(unsigned *p, unsigned x) { atomicAdd(
 // All steps of a network of at most kOwn * LANES neurons, by a block (LANES =
 // 256) or a warp (32).  A step of the general form below is five dependent
 // trips to memory: state and parameters, event range, row bounds, synapses, and
-// the stores in between.  Here a thread keeps the state, the parameters and the
-// row bounds of its neurons in registers, a spiker's list entry carries its row,
-// and the external input of t + 1 is prepared while the first synapses of step t
-// are on their way: one trip a step, 4.6 -> 2.5 us
-// at 1021 neurons with two blocks an SM.  What bounds it now is the instruction
+// the stores in between.  Here a thread keeps the state and the parameters of its
+// neurons in registers, a spiker's list entry carries its row, and the external
+// input of t + 1 is prepared while the first synapses of step t are on their way:
+// one trip a step, 4.6 -> 2.5 us at 1021 neurons with two blocks an SM.  What bounds it now is the instruction
 // issue of an SM's 16 warps (the draws' 64-bit multiplies, the rule, the synapses).
 // `list` holds kOwn * LANES rows and `rows` as many; `cnt` two counters, both
 // zero.  (The row bounds lie in shared memory and the amplitudes, which few
@@ -533,7 +532,13 @@ cudaError_t max_grid_batch(int dtype, bool own, int ring_smem, int *grid) {
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const size_t smem = batch_smem(ring_smem);
-    e = cudaFuncSetAttribute(batch_fn(dtype, own), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is the function's, shared by every context of the process: always
+    // the device's largest, so that a context with a smaller ring does not lower
+    // it under another's graph
+    int lim = 0;
+    e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(batch_fn(dtype, own), cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_fn(dtype, own), kBatchBlock, smem);
     if (e != cudaSuccess) return e;

@@ -75,8 +75,6 @@ sn_status batch_run(sn_ctx *c, int steps) {
     kp.sharedMemBytes = (unsigned)batch_smem(c->ring_smem);
     kp.kernelParams = args;
     if (!c->graph_exec) {
-        SN_CUDA(c, cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)kp.sharedMemBytes));
         SN_CUDA(c, cudaGraphCreate(&c->graph, 0));
         cudaMemsetParams mp;
         memset(&mp, 0, sizeof(mp));

@@ -60,3 +60,19 @@ def test_same_bits_as_the_general_form(config, integer):
         assert np.array_equal(x, y), f"network {b} of {len(nets[b]['threshold'])} neurons"
     assert np.array_equal(np.asarray(v).view(np.int32), np.asarray(v0)[:len(v)].view(np.int32))
     assert np.array_equal(r, np.asarray(r0)[:len(r)])
+
+
+def test_two_contexts_with_different_rings():
+    """The shared-memory limit of the kernel is the process's: a second context
+    with a smaller ring leaves the first one's graph launchable."""
+    from paper_2305_02510_gb300 import sn as S
+    nets = networks(True)[:6]
+    a = S.from_batch_workloads(nets, record_steps=60)
+    S.sn_batch_config(a, 0, 160 * 1024)
+    S.sn_run(a, 10)
+    b = S.from_batch_workloads(nets, record_steps=60)
+    S.sn_batch_config(b, 0, 0)
+    S.sn_run(b, 10)
+    S.sn_run(a, 7)
+    S.sn_run(b, 7)
+    assert np.array_equal(S.sn_get_spikes(a, 0, 17), S.sn_get_spikes(b, 0, 17))
