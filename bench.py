@@ -32,6 +32,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "synaptic events/s & timesteps/s on 1 GB300 (batched vs plain); BPTT step ms"
 UNIT = "synaptic events/s"
+PULL_KERNEL = "pull_block_kernel<SN_F32>"      # the benchmark network's pull form
 TIMESTEPS = 1000
 # per-neuron state bytes touched once per timestep by the update phase:
 # V and r read+write (16), threshold/leak/reset/refractory/Poisson rate and
@@ -46,10 +47,13 @@ STATE_BYTES_PULL = 40
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.txt")
 CSRC = os.path.join(ROOT, "paper_2305_02510_gb300", "csrc")
 KERNEL_SOURCES = {
+    "pull_block_kernel": ["sn_pull_block.cu", "sn_pull.cuh", "sn_device.cuh", "sn_internal.h"],
     "sparse_pull_kernel": ["sn_pull.cu", "sn_device.cuh", "sn_internal.h"],
     "sparse_reg_kernel": ["sn_kernels.cu", "sn_device.cuh", "sn_internal.h"],
     "dense_kernel": ["sn_kernels.cu", "sn_device.cuh", "sn_internal.h"],
     "batch_kernel": ["sn_batch.cu", "sn_device.cuh", "sn_internal.h"],
+    "dense_res_kernel": ["sn_dense_res.cu", "sn_device.cuh", "sn_internal.h"],
+    "shared_res_kernel": ["sn_shared_res.cu", "sn_shared.cuh", "sn_tc.cuh", "sn_device.cuh", "sn_internal.h"],
     "shared_kernel": ["sn_shared.cu", "sn_tc.cuh", "sn_device.cuh", "sn_internal.h"],
 }
 
@@ -511,7 +515,7 @@ def bptt_extra(S, W, torch, stream):
                         "checkpoint every 10", "synapses": syn, "ms_per_training_step": ms,
             "roofline": {"bound": "tensor", "achieved": alg / (ms / 1e3) / 1e12, "peak": bf16, "unit": "TFLOP/s",
                          "frac": alg / (ms / 1e3) / 1e12 / bf16, "peak_source": src,
-                         "kernel": "ff_tc_fwd_kernel + ff_tc_kernel (whole step's work over the step time)",
+                         "kernel": "ff_tc_rows_kernel + ff_tc_dw_kernel (whole step's work over the step time)",
                          "algorithmic_flop_per_step": alg,
                          "executed_tensor_flop_per_step": flop,
                          "executed_frac": flop / (ms / 1e3) / 1e12 / bf16,
@@ -559,7 +563,7 @@ def shared_extra(S, W, torch, stream, flush):
             "ms": ms, "synaptic_events_per_s": ev / (ms / 1e3), "spikes_per_train_step": spk / (B * T),
             "roofline": {"bound": "tensor", "achieved": ops / (ms / 1e3) / 1e12, "peak": peak,
                          "unit": "TFLOP/s", "frac": ops / (ms / 1e3) / 1e12 / peak, "peak_source": src,
-                         "kernel": "shared_kernel (tcgen05.mma kind::f8f6f4)"},
+                         "kernel": "shared_res_kernel (tcgen05.mma kind::f8f6f4)"},
             "plain_ms": total, "plain_synaptic_events_per_s": pev / (total / 1e3),
             "speedup_vs_plain": total / ms, "launches": 1, "plain_launches": B}
 
@@ -806,7 +810,7 @@ def main():
         # synapse every step, which is reported beside it
         abytes = event_bytes(n, T, spikes, events)
         form_bytes = algorithmic_bytes_pull(n, m, T) if pull else algorithmic_bytes(n, T, spikes, events)
-        kernel = "sparse_pull_kernel<SN_F32>" if pull else "sparse_reg_kernel<SN_F32>"
+        kernel = PULL_KERNEL if pull else "sparse_reg_kernel<SN_F32>"
         achieved = abytes / (ms / 1e3) / 1e9
         traffic, traffic_src = recorded_traffic(kernel, f"large-sparse T={T}")
         store = None
@@ -834,14 +838,15 @@ def main():
                                         "event (synapse + accumulate), 56 B state and a raster bit per "
                                         "neuron and timestep",
                          "pull_store": store,
-                         "kernel_bound": (f"l2+barrier: the pull store of incoming synapses "
-                                          f"({store['bytes'] / 1e6:.0f} MB) stays in the L2; each timestep "
-                                          f"streams it from L2 once, then one grid barrier")
+                         "kernel_bound": (f"issue: the pull store of incoming synapses "
+                                          f"({store['bytes'] / 1e6:.0f} MB) stays in the L2; its synapses of "
+                                          f"delay 4 and more are looked up once per three timesteps, and "
+                                          f"blocks wait for one another's spike words every timestep")
                                          if pull else "l2 atomics: scattered accumulates into the pending-input "
                                                       "ring, L2-resident",
                          "form_bytes_per_launch": form_bytes,
                          "frac_form_bytes": form_bytes / (ms / 1e3) / 1e9 / peak,
-                         "form_bytes_model": "pull: 8 B per synapse every timestep + 40 B state and a raster "
+                         "form_bytes_model": "pull, step by step: 8 B per synapse every timestep + 40 B state and a raster "
                                              "bit per neuron and timestep" if pull else "push: as above"},
             "e2e": {"value": e2e_ev_all / e2e_all, "unit": UNIT,
                     "h2d_bytes_per_step": 8 * n,
@@ -857,7 +862,7 @@ def main():
                 o_bytes = algorithmic_bytes(n, T, o_spk, o_ev) if pull else algorithmic_bytes_pull(n, m, T)
                 alt = {"propagation": "push" if pull else "pull", "ms_per_step": o_ms,
                        "value": o_ev / (o_ms / 1e3), "unit": UNIT,
-                       "kernel": "sparse_reg_kernel<SN_F32>" if pull else "sparse_pull_kernel<SN_F32>",
+                       "kernel": "sparse_reg_kernel<SN_F32>" if pull else PULL_KERNEL,
                        "roofline_frac": o_bytes / (o_ms / 1e3) / 1e9 / peak}
             except S.SnError as e:
                 alt = {"unavailable": str(e)}

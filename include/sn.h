@@ -108,9 +108,12 @@ typedef enum {
 #define SN_PULL_CODED 0x2000u
                             /* sn_create only: the form of the pull store (see
                                sn_pull_store_info).  Without either flag the
-                               library builds the plain form while it takes at
-                               most 80 % of the L2 cache, else the smaller
-                               form.  The two forms
+                               library builds the plain form, ordered for
+                               blocks of three steps; for a network of one
+                               block of threads, or lists that form cannot
+                               count, the plain form while it takes at most
+                               80 % of the L2 cache, else the smaller form.
+                               The forms
                                hold the same synapses in the same order, so
                                the results are identical; the flags let tests
                                and tuning run either                          */

@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kBlock, AHEAD ? 5 : 0) sparse_kernel(NetArgs a
             // runs while the barrier's arrivals come in, two synapses a lane at a
             // time; only the spike bits are read after it.  (Rows after the barrier,
             // then columns, one synapse a lane: 15.5 us a step at 10,007 neurons
-            // of 50 synapses; 12.6 so.)
+            // of 50 synapses; 12.9 so.)
             constexpr int U = 2;
             const unsigned *rrow = a.raster + (size_t)(t % a.cap) * a.words;
             const float *xo = a.trace + (size_t)((t & 1) ^ 1) * a.n;

@@ -1,7 +1,7 @@
 """Dense networks small enough for their weights to stay in shared memory: a run
-in launches long enough for that form (4 steps, 12 with plasticity) leaves the same spikes and the same saved
-state, byte for byte (voltages, refractory counters, pending input, spike words,
-weights, traces), as the same run in launches of at most three steps, which
+in launches long enough for that form (4 steps, 12 with plasticity) leaves the
+same spikes and the same saved state, byte for byte (voltages, refractory
+counters, pending input, spike words, weights, traces), as the same run in launches of at most three steps, which
 stream the rows from memory.  Sizes at the edges of a warp, of one block, of the
 vector form (n % 4 == 0) and of the shared memory (the largest with and without
 plasticity, and the first size past each, where both runs stream)."""
