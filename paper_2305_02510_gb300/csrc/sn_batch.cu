@@ -532,14 +532,7 @@ cudaError_t max_grid_batch(int dtype, bool own, int ring_smem, int *grid) {
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const size_t smem = batch_smem(ring_smem);
-    // the limit is the function's, shared by every context of the process: always
-    // the device's largest, so that a context with a smaller ring does not lower
-    // it under another's graph
-    int lim = 0;
-    e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(batch_fn(dtype, own), cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-    if (e != cudaSuccess) return e;
+    if ((e = allow_all_smem(batch_fn(dtype, own))) != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_fn(dtype, own), kBatchBlock, smem);
     if (e != cudaSuccess) return e;
     *grid = per * sms;

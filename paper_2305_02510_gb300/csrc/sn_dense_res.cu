@@ -404,14 +404,9 @@ size_t dense_tag_bytes(int n) {
 }
 
 cudaError_t launch_dense_res(const NetArgs &a, int grid, cudaStream_t s) {
-    int dev = 0, lim = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess) return e;
     const bool vec = a.n % 4 == 0 && ((uintptr_t)a.W & 15u) == 0;
     const void *fn = res_fn(a.chunk / 32, a.stdp != 0, vec);
-    // the same limit for every network: another thread's launch cannot lower it
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
+    cudaError_t e = allow_all_smem(fn);
     if (e != cudaSuccess) return e;
     if (grid > 1) {
         dense_tag_init_kernel<<<1, 256, 0, s>>>(a.ptag, 2 * a.words * kDenseTagStride);

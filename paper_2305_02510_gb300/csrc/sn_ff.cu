@@ -590,8 +590,7 @@ cudaError_t ff_dw(const float *gI, const unsigned *sprev, int words_in, const ui
                   int B, int T, int splits, float *part, float *dW, cudaStream_t s) {
     if (T * B <= kDwSparseMaxRows) {
         const size_t smem = (size_t)T * B * sizeof(int);
-        cudaError_t e = cudaFuncSetAttribute((const void *)ff_dw_sparse_kernel,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_all_smem((const void *)ff_dw_sparse_kernel);
         if (e != cudaSuccess) return e;
         dim3 g(n_in, (n_out + kDwCols - 1) / kDwCols);
         ff_dw_sparse_kernel<<<g, 256, smem, s>>>(gI, sprev, words_in, D, n_in, n_out, B, T, dW);

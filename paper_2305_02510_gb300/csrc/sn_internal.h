@@ -13,6 +13,20 @@
 
 namespace sn {
 
+// The limit on a kernel's dynamic shared memory is the function's, shared by every
+// context and thread of the process.  It is set to all that a block may have, never
+// to one network's bytes: a smaller network planned or launched by another thread
+// between a set and its launch would lower it under that launch.
+inline cudaError_t allow_all_smem(const void *fn) {
+    int dev = 0, lim = 0;
+    cudaFuncAttributes at;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - (int)at.sharedSizeBytes);
+}
+
 enum Kind { KIND_SPARSE = 0, KIND_DENSE = 1, KIND_BATCH = 2, KIND_SHARED_I8 = 3, KIND_FF = 4 };
 
 // Grid barrier state (one per context): the arrival count of the running

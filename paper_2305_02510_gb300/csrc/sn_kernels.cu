@@ -491,7 +491,7 @@ cudaError_t launch_sparse(const NetArgs &a, int dtype, int grid, int block, cuda
     else
         fn = (const void *)sparse_kernel<SN_I32, false>;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_all_smem(fn);
         if (e != cudaSuccess) return e;
     }
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, smem, s);
@@ -982,8 +982,6 @@ cudaError_t launch_dense(const NetArgs &a, int grid, int block, cudaStream_t s) 
     const void *fn = dense_fn(a.chunk / 32, a.stdp != 0, vec);
     cudaError_t e = reset_barrier(a.ctl, s);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kBlock), args, smem, s);
 }
 
@@ -1004,8 +1002,7 @@ cudaError_t plan_dense(int n, int *grid, int *chunk, int force_cpl) {
         int per = 1 << 30;
         for (int v = 0; v < 3; ++v) {
             const void *fn = dense_fn(cpl, v == 1, v == 2);
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
+            if ((e = allow_all_smem(fn)) != cudaSuccess) return e;
             int p = 0;
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, fn, kBlock, smem);
             if (e != cudaSuccess) return e;

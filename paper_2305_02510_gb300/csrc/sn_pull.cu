@@ -477,8 +477,7 @@ cudaError_t plan_pull(int n, int D, long long m, int *grid, int *chunk, int *row
     const int block = (int)(per * 32);
     for (const void *fn : {pull_fn(SN_F32, false), pull_fn(SN_I32, false), pull_fn(SN_F32, true),
                            pull_fn(SN_I32, true)}) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
+        if ((e = allow_all_smem(fn)) != cudaSuccess) return e;
         int p = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, fn, block, (size_t)bytes);
         if (e != cudaSuccess) return e;
@@ -496,8 +495,6 @@ cudaError_t launch_sparse_pull(const NetArgs &a, int dtype, bool coded, int grid
     const void *fn = pull_fn(dtype, coded);
     // the grid barrier's arrival count starts every launch at zero
     cudaError_t e = cudaMemsetAsync(&a.ctl->bar, 0, sizeof(GridBarrier), s);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(a.chunk), args, smem, s);
 }

@@ -568,7 +568,7 @@ cudaError_t plan_pull_block(int n, int D, int dtype, int grid, int chunk, int *h
     const size_t bytes = (D > 3 ? (words + (words & 1)) * bits * 4 : 0) + 2 * wp * 4 + (size_t)chunk * 4;
     if (bytes + 1100 > (size_t)optin || grid > sms || (words + 1) / 2 > (size_t)kCols * chunk) return cudaSuccess;
     const void *fn = block_fn(dtype, bits, chunk);
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if ((e = allow_all_smem(fn)) != cudaSuccess) return e;
     int p = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, fn, chunk, bytes)) != cudaSuccess) return e;
     if (p < 1) return cudaSuccess;
@@ -597,8 +597,6 @@ cudaError_t launch_pull_block(NetArgs a, int dtype, int hb, int grid, size_t sme
     const int total = kTagRows * a.wt;
     pull_tag_init_kernel<<<(total + 255) / 256, 256, 0, s>>>(a);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // cooperative: the blocks wait for one another's rows, so all must be resident
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(a.chunk), args, smem, s);
