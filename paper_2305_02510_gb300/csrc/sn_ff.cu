@@ -234,6 +234,10 @@ __global__ void __launch_bounds__(kScanBlock) ff_scan_fwd_kernel(const float *__
 // the adjoint: those of segment sg - 1 are copied into the thread's own
 // column of a shared-memory buffer (asynchronous 4-byte copies) while segment
 // sg is computed, and its checkpoint is loaded into registers.
+// With gbf, more threads (columns n .. ldg - 1) zero the padding of its rows: the
+// buffer is shared by the layers, and what another one left there may be an Inf or a
+// NaN, which the contraction's zero weights would not cancel.  (Tensor maps that end
+// at the true width do the same, but took a step at 700-1024-1024-20 13 us longer.)
 constexpr int kBwdBlock = 128;
 
 template <int K>
@@ -243,7 +247,14 @@ __global__ void __launch_bounds__(kBwdBlock) ff_scan_bwd_kernel(const float *__r
                                    float *__restrict__ gI, __nv_bfloat16 *__restrict__ gbf, int ldg) {
     __shared__ float sI[2][K][kBwdBlock], sG[2][K][kBwdBlock];
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (tid >= (long long)B * n) return;
+    if (tid >= (long long)B * n) {
+        const int pad = ldg - n;
+        const long long q = tid - (long long)B * n;
+        if (!gbf || q >= (long long)B * pad) return;
+        for (size_t r = (size_t)(q / pad); r < (size_t)2 * T * B; r += B)
+            gbf[r * ldg + n + q % pad] = __float2bfloat16_rn(0.0f);
+        return;
+    }
     const int b = (int)(tid / n), j = (int)(tid - (long long)(tid / n) * n);
     const int segs = (T + K - 1) / K;
     const float gcount = gc ? gc[(size_t)b * n + j] : 0.0f;
@@ -565,7 +576,7 @@ cudaError_t ff_scan_bwd(const float *I, int n, int B, int T, int k, float theta,
                         int refractory, float slope, const float *vck, const int *rck, const float *gs,
                         const float *gc, float *gI, void *gbf, int ldg, cudaStream_t s) {
     FFNeuron p{theta, leak, reset, slope, refractory};
-    const long long threads = (long long)B * n;
+    const long long threads = (long long)B * (gbf ? ldg : n);
     const int nb = blocks_for(threads, kBwdBlock);
     __nv_bfloat16 *g2 = (__nv_bfloat16 *)gbf;
     switch (k) {

@@ -22,14 +22,11 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 
 inline int up(int x, int m) { return (x + m - 1) / m * m; }
 
-// Row-major BF16 [rows][cols], a row every up(cols, 64) elements, boxes of box_rows
-// rows x 64 columns, 128-byte swizzle; coordinates outside the tensor read as zero.
-// The map ends at the true width: the buffers are shared by layers and passes, and
-// what lies in a row's padding is another one's, perhaps an Inf or a NaN, which a
-// zero weight would not cancel.
-sn_status bf16_map(sn_ctx *c, CUtensorMap *out, const void *base, long long rows, int cols, int box_rows = 128) {
+// Row-major BF16 [rows][cols] (cols a multiple of 64), boxes of box_rows rows x 64
+// columns, 128-byte swizzle; coordinates outside the tensor read as zero.
+sn_status bf16_map(sn_ctx *c, CUtensorMap *out, const void *base, long long rows, long long cols, int box_rows = 128) {
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)up(cols, 64) * 2};
+    cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
     cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     cuuint32_t es[2] = {1, 1};
     CUresult r = ((EncodeTiledFn)c->ff_encode)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)base, dims, strides,
@@ -54,8 +51,8 @@ sn_status tc_forward(sn_ctx *c, int l, float *I) {
     memset(&a, 0, sizeof(a));
     sn_status s;
     a.bn = nout < 128 ? up(nout, 16) : 128;
-    if ((s = bf16_map(c, &maps.m[0], c->ff_Sbf[l - 1], rows, nin)) ||
-        (s = bf16_map(c, &maps.m[2], c->ff_Wf[l - 1], 12LL * rows_out, nin, a.bn)))
+    if ((s = bf16_map(c, &maps.m[0], c->ff_Sbf[l - 1], rows, nin_p)) ||
+        (s = bf16_map(c, &maps.m[2], c->ff_Wf[l - 1], 12LL * rows_out, nin_p, a.bn)))
         return s;
     a.M = rows; a.N = nout; a.kblocks = nin_p / 64; a.shift = -B; a.part_rows = rows_out;
     a.C = I; a.ldc = nout; a.ctl = c->ctl;
@@ -77,9 +74,9 @@ sn_status tc_weight_grad(sn_ctx *c, int l, float *dW) {
     memset(&a, 0, sizeof(a));
     sn_status s;
     const __nv_bfloat16 *G = (const __nv_bfloat16 *)c->ff_G;
-    if ((s = bf16_map(c, &maps.m[0], c->ff_Sbf[l - 1], rows, nin, 64)) ||
-        (s = bf16_map(c, &maps.m[1], G, rows, nout, 64)) ||
-        (s = bf16_map(c, &maps.m[2], G + (size_t)rows * nout_p, rows, nout, 64)))
+    if ((s = bf16_map(c, &maps.m[0], c->ff_Sbf[l - 1], rows, up(nin, 64), 64)) ||
+        (s = bf16_map(c, &maps.m[1], G, rows, nout_p, 64)) ||
+        (s = bf16_map(c, &maps.m[2], G + (size_t)rows * nout_p, rows, nout_p, 64)))
         return s;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
@@ -119,9 +116,9 @@ sn_status tc_spike_grad(sn_ctx *c, int l) {
     sn_status s;
     const __nv_bfloat16 *G = (const __nv_bfloat16 *)c->ff_G;
     a.bn = nin < 128 ? up(nin, 16) : 128;
-    if ((s = bf16_map(c, &maps.m[0], G, rows, nout)) ||
-        (s = bf16_map(c, &maps.m[1], G + (size_t)rows * nout_p, rows, nout)) ||
-        (s = bf16_map(c, &maps.m[2], c->ff_Wb[l - 1], 8LL * rows_in, nout, a.bn)))
+    if ((s = bf16_map(c, &maps.m[0], G, rows, nout_p)) ||
+        (s = bf16_map(c, &maps.m[1], G + (size_t)rows * nout_p, rows, nout_p)) ||
+        (s = bf16_map(c, &maps.m[2], c->ff_Wb[l - 1], 8LL * rows_in, nout_p, a.bn)))
         return s;
     a.M = rows; a.N = nin; a.kblocks = nout_p / 64; a.shift = B; a.part_rows = rows_in;
     a.C = c->ff_gS; a.ldc = nin; a.ctl = c->ctl;
@@ -151,9 +148,9 @@ void tc_setup(sn_ctx *c) {
         const size_t wf = (size_t)12 * up(nout, 128) * up(nin, 64) * 2, wb = (size_t)8 * up(nin, 128) * up(nout, 64) * 2;
         if (dalloc(c, &c->ff_Wf[l - 1], wf) || dalloc(c, &c->ff_Wb[l - 1], wb))
             return;
-        // the weight parts of the other three delays stay zero for the
-        // context's lifetime (each forward rewrites only every weight's own
-        // delay slot)
+        // the weight parts of the other three delays and the padding stay
+        // zero for the context's lifetime (each forward rewrites only every
+        // weight's own delay slot)
         if (cudaMemset(c->ff_Wf[l - 1], 0, wf) || cudaMemset(c->ff_Wb[l - 1], 0, wb)) return;
     }
     // The spike operand of every layer stays for the weight gradient, like the
@@ -164,9 +161,11 @@ void tc_setup(sn_ctx *c) {
     for (int l = 0; l < L; ++l) {
         if (l > 0 && c->ff_S_shared) { c->ff_Sbf[l] = c->ff_Sbf[0]; continue; }
         const size_t bytes = (c->ff_S_shared ? s_elems : (size_t)rows * up(c->ff_sizes[l], 64)) * 2;
-        if (dalloc(c, &c->ff_Sbf[l], bytes)) return;
+        // padding columns stay zero (in a shared buffer they may later hold 0/1
+        // values of a wider layer, which meet zero weight columns)
+        if (dalloc(c, &c->ff_Sbf[l], bytes) || cudaMemset(c->ff_Sbf[l], 0, bytes)) return;
     }
-    if (dalloc(c, &c->ff_G, g_elems * 2)) return;
+    if (dalloc(c, &c->ff_G, g_elems * 2) || cudaMemset(c->ff_G, 0, g_elems * 2)) return;
     c->ff_tc_ok = true;
 }
 
