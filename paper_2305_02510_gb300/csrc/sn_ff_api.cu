@@ -127,16 +127,36 @@ sn_status tc_spike_grad(sn_ctx *c, int l) {
     return SN_OK;
 }
 
-// Allocate the BF16 operand buffers and look up the tensor-map encoder; on
-// any failure the context keeps the SIMT engine only.
-void tc_setup(sn_ctx *c) {
+// Spike operands of layers 0 .. L-1: a buffer each, or one for all of them that
+// holds s_elems.  False, with nothing held, when the memory is not there.
+bool tc_spike_operands(sn_ctx *c, bool shared, size_t s_elems) {
+    const int L = c->ff_layers, rows = c->ff_batch * c->ff_steps;
+    c->ff_S_shared = shared;
+    c->ff_Sbf.assign(L, nullptr);
+    for (int l = 0; l < L; ++l) {
+        if (l > 0 && shared) { c->ff_Sbf[l] = c->ff_Sbf[0]; continue; }
+        const size_t bytes = (shared ? s_elems : (size_t)rows * up(c->ff_sizes[l], 64)) * 2;
+        // padding columns stay zero (in a shared buffer they may later hold 0/1
+        // values of a wider layer, which meet zero weight columns)
+        if (dalloc(c, &c->ff_Sbf[l], bytes) || cudaMemset(c->ff_Sbf[l], 0, bytes)) {
+            for (void *q : c->ff_Sbf) dfree(c, q);
+            c->ff_Sbf.assign(L, nullptr);
+            return false;
+        }
+    }
+    return true;
+}
+
+// Allocate the BF16 operand buffers and look up the tensor-map encoder; false (and
+// the context keeps the SIMT engine only) when they cannot be had.
+bool tc_buffers(sn_ctx *c) {
     const int L = c->ff_layers, B = c->ff_batch, rows = B * c->ff_steps;
-    if (B % 8 != 0) return;
+    if (B % 8 != 0) return false;
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
         q != cudaDriverEntryPointSuccess || !fn)
-        return;
+        return false;
     c->ff_encode = fn;
     size_t s_elems = 0, g_elems = 0;
     c->ff_Wf.assign(L, nullptr);
@@ -147,26 +167,28 @@ void tc_setup(sn_ctx *c) {
         g_elems = std::max(g_elems, (size_t)2 * rows * up(nout, 64));
         const size_t wf = (size_t)12 * up(nout, 128) * up(nin, 64) * 2, wb = (size_t)8 * up(nin, 128) * up(nout, 64) * 2;
         if (dalloc(c, &c->ff_Wf[l - 1], wf) || dalloc(c, &c->ff_Wb[l - 1], wb))
-            return;
+            return false;
         // the weight parts of the other three delays and the padding stay
         // zero for the context's lifetime (each forward rewrites only every
         // weight's own delay slot)
-        if (cudaMemset(c->ff_Wf[l - 1], 0, wf) || cudaMemset(c->ff_Wb[l - 1], 0, wb)) return;
+        if (cudaMemset(c->ff_Wf[l - 1], 0, wf) || cudaMemset(c->ff_Wb[l - 1], 0, wb)) return false;
     }
+    if (dalloc(c, &c->ff_G, g_elems * 2)) return false;
     // The spike operand of every layer stays for the weight gradient, like the
-    // synaptic input; a context that recomputes that also expands the spikes
-    // again, into one buffer.
-    c->ff_S_shared = c->ff_Ik.empty();
-    c->ff_Sbf.assign(L, nullptr);
-    for (int l = 0; l < L; ++l) {
-        if (l > 0 && c->ff_S_shared) { c->ff_Sbf[l] = c->ff_Sbf[0]; continue; }
-        const size_t bytes = (c->ff_S_shared ? s_elems : (size_t)rows * up(c->ff_sizes[l], 64)) * 2;
-        // padding columns stay zero (in a shared buffer they may later hold 0/1
-        // values of a wider layer, which meet zero weight columns)
-        if (dalloc(c, &c->ff_Sbf[l], bytes) || cudaMemset(c->ff_Sbf[l], 0, bytes)) return;
-    }
-    if (dalloc(c, &c->ff_G, g_elems * 2) || cudaMemset(c->ff_G, 0, g_elems * 2)) return;
-    c->ff_tc_ok = true;
+    // synaptic input; a context that recomputes that, or has no memory for them
+    // all, expands the spikes again, into one buffer.
+    return (!c->ff_Ik.empty() && tc_spike_operands(c, false, s_elems)) || tc_spike_operands(c, true, s_elems);
+}
+
+void tc_setup(sn_ctx *c) {
+    c->ff_tc_ok = tc_buffers(c);
+    if (c->ff_tc_ok) return;
+    for (void *q : c->ff_Wf) dfree(c, q);
+    for (void *q : c->ff_Wb) dfree(c, q);
+    dfree(c, c->ff_G);
+    c->ff_Wf.clear();
+    c->ff_Wb.clear();
+    c->ff_G = nullptr;
 }
 
 }  // namespace
