@@ -189,11 +189,11 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
     // TMEM go away (bounded waits; no-ops when the phases have completed)
     if (warp == 0 && lane == 0) {
         for (unsigned i = g_prod > kDwSt ? g_prod - kDwSt : 0; i < g_prod; ++i)
-            mbar_wait(smem_addr(&full[i % kDwSt]), (i / kDwSt) & 1u, a.ctl);
+            mbar_drain(smem_addr(&full[i % kDwSt]), (i / kDwSt) & 1u);
     }
     if (warp == 1 && lane == 0) {
         for (unsigned i = g_mma > kDwSt ? g_mma - kDwSt : 0; i < g_mma; ++i)
-            mbar_wait(smem_addr(&empty[i % kDwSt]), (i / kDwSt) & 1u, a.ctl);
+            mbar_drain(smem_addr(&empty[i % kDwSt]), (i / kDwSt) & 1u);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
     using R = Rows<H, SG>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t fullA[R::RA], emptyA[R::RA], fullB[R::RB], emptyB[R::RB], accf[2], acce[2];
+    __shared__ __align__(8) uint64_t fullA[R::RA], emptyA[R::RA], fullB[R::RB], emptyB[R::RB], accf[2], acce[2], mmas_done;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -252,6 +252,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
         for (int q = 0; q < R::RA; ++q) { init(&fullA[q], 1); init(&emptyA[q], 1); }
         for (int q = 0; q < R::RB; ++q) { init(&fullB[q], 1); init(&emptyB[q], 1); }
         for (int q = 0; q < 2; ++q) { init(&accf[q], 1); init(&acce[q], 8); }
+        init(&mmas_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         s_abort = 0;
@@ -433,13 +434,14 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
     // TMEM go away (bounded waits; no-ops when the phases have completed)
     if (warp == 0 && lane == 0) {
         for (unsigned i = ua > R::RA ? ua - R::RA : 0; i < ua; ++i)
-            mbar_wait(smem_addr(&fullA[i % R::RA]), (i / R::RA) & 1u, a.ctl);
+            mbar_drain(smem_addr(&fullA[i % R::RA]), (i / R::RA) & 1u);
         for (unsigned i = ub > R::RB ? ub - R::RB : 0; i < ub; ++i)
-            mbar_wait(smem_addr(&fullB[i % R::RB]), (i / R::RB) & 1u, a.ctl);
+            mbar_drain(smem_addr(&fullB[i % R::RB]), (i / R::RB) & 1u);
     }
-    if (warp == 1 && lane == 0) {
-        for (unsigned i = ua > R::RA ? ua - R::RA : 0; i < ua; ++i)
-            mbar_wait(smem_addr(&emptyA[i % R::RA]), (i / R::RA) & 1u, a.ctl);
+    if (warp == 1) {
+        // (every MMA issued, also those of a step that a failed wait cut short)
+        mma_commit(smem_addr(&mmas_done));
+        mbar_drain(smem_addr(&mmas_done), 0);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();

@@ -244,11 +244,11 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
     // phases have already completed)
     if (warp == 0 && lane == 0) {
         for (unsigned i = g_prod > kStages ? g_prod - kStages : 0; i < g_prod; ++i)
-            mbar_wait(smem_addr(&full[i % kStages]), (i / kStages) & 1u, a.ctl);
+            mbar_drain(smem_addr(&full[i % kStages]), (i / kStages) & 1u);
     }
     if (warp == 1 && lane == 0) {
         for (unsigned i = g_mma > kStages ? g_mma - kStages : 0; i < g_mma; ++i)
-            mbar_wait(smem_addr(&empty[i % kStages]), (i / kStages) & 1u, a.ctl);
+            mbar_drain(smem_addr(&empty[i % kStages]), (i / kStages) & 1u);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();

@@ -294,7 +294,7 @@ shared_res_kernel(const __grid_constant__ CUtensorMap tmW, SharedArgs a) {
             }
         // loads in flight land before the block's shared memory goes away
         for (unsigned i = issued > kStagesW ? issued - kStagesW : 0; i < issued; ++i)
-            mbar_wait(smem_addr(&fullW[i % kStagesW]), (i / kStagesW) & 1u, a.ctl);
+            mbar_drain(smem_addr(&fullW[i % kStagesW]), (i / kStagesW) & 1u);
     } else if (warp == kOwners + 1) {
         // MMAs; the next barriers are looked at before those at hand are issued
         constexpr uint32_t idesc = idesc_e4m3_f32(kTM, kTN);
@@ -322,7 +322,7 @@ shared_res_kernel(const __grid_constant__ CUtensorMap tmW, SharedArgs a) {
         }
         // MMAs issued complete before TMEM goes away
         for (unsigned i = issued > kStagesA ? issued - kStagesA : 0; i < issued; ++i)
-            mbar_wait(smem_addr(&emptyA[i % kStagesA]), (i / kStagesA) & 1u, a.ctl);
+            mbar_drain(smem_addr(&emptyA[i % kStagesA]), (i / kStagesA) & 1u);
     }
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");

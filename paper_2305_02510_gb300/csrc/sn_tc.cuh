@@ -55,6 +55,17 @@ __device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, Control *ctl) {
     }
 }
 
+// Wait before shared memory or TMEM goes away, for a phase that copies or MMAs in
+// flight will complete: bounded by the wall clock alone, whatever status is latched.
+__device__ inline void mbar_drain(uint32_t bar, uint32_t parity) {
+    unsigned long long t0 = 0;
+    while (!mbar_try(bar, parity)) {
+        const unsigned long long now = global_timer_ns();
+        if (t0 == 0) t0 = now;
+        else if (now - t0 > kWaitNs) return;
+    }
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
