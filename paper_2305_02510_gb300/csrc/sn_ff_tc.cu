@@ -94,7 +94,8 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
     bool ready = false;                            // the next stage's operands are known to be there
     const int items = a.tiles_m * a.tiles_n * a.ksplit;
 
-    for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+    bool live = true;                              // no wait of this block has given up (the same for all threads)
+    for (int item = blockIdx.x; item < items && live; item += gridDim.x) {
         const int ks = item % a.ksplit, tile = item / a.ksplit;
         const int tm = tile % a.tiles_m, tn = tile / a.tiles_m;
         const int kb0 = (int)((long long)a.kblocks * ks / a.ksplit);
@@ -121,8 +122,7 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
         } else if (warp == 1) {
             for (int kb = kb0; kb < kb1; ++kb, ++g_mma) {
                 const int st = g_mma % kDwSt;
-                if (!ready && !mbar_wait(smem_addr(&full[st]), (g_mma / kDwSt) & 1u, a.ctl)) { s_abort = 1; break; }
-                ready = mbar_test(smem_addr(&full[(g_mma + 1) % kDwSt]), ((g_mma + 1) / kDwSt) & 1u);
+                if (!ready && !mbar_wait_warp(smem_addr(&full[st]), (g_mma / kDwSt) & 1u, a.ctl)) { s_abort = 1; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint64_t d0 = umma_desc_mn_sw128(sbase + st * kDwStageBytes, kDwHalf);
 #pragma unroll
@@ -131,14 +131,15 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
                     mma_bf16_x4<128>(tmem + d * kT, d0 + (2 + d) * (kDwTile / 16), d0 + kDwTile / 16, idesc, 1);
                 }
                 mma_commit(smem_addr(&empty[st]));
+                ready = mbar_test_warp(smem_addr(&full[(g_mma + 1) % kDwSt]), ((g_mma + 1) / kDwSt) & 1u);
             }
             mma_commit(smem_addr(&accbar));
         }
         __syncwarp();
-        const bool ok = mbar_wait(smem_addr(&accbar), items_done & 1u, a.ctl);
+        if (!mbar_wait(smem_addr(&accbar), items_done & 1u, a.ctl)) s_abort = 1;
         ++items_done;
-        if (!ok) s_abort = 1;
         __syncthreads();
+        live = !s_abort;                           // (nobody sets it before the item's last barrier)
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         // epilogue: warps w and w + 4 read TMEM lane quarter w (tile rows), each
         // half of the columns, every element from its own delay's accumulator;
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
             for (int d = 0; d < 4; ++d) {
                 uint32_t v[32];
                 tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(d * kT + c0), v);
-                if (!ok || kb1 == kb0 || m >= a.M) continue;
+                if (!live || kb1 == kb0 || m >= a.M) continue;
                 const uint8_t *Dr = a.D + (size_t)m * a.N;
 #pragma unroll
                 for (int q = 0; q < 32; ++q)
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
                 dst[q4] = make_float4(out[4 * q4], out[4 * q4 + 1], out[4 * q4 + 2], out[4 * q4 + 3]);
         }
         __syncthreads();
-        if (ok) {
+        if (live) {
             float *C = a.C + (size_t)ks * a.cstride;
             const int ncol = min(kT, a.N - tn * kT);
             for (int row = warp; row < kT; row += kThreads / 32) {
@@ -307,24 +308,25 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
         const uint32_t idesc = idesc_bf16_f32(kT, a.bn);
         const uint64_t descA = umma_desc_sw128(baseA), descB = umma_desc_sw128(baseB);
         unsigned g_chunk = 0;
-        // barriers are looked at before the MMAs in front of theirs go out
+        // barriers are looked at while the MMAs in front of theirs run
         bool seenA = false, seenB = false;
         auto waitA = [&](unsigned u) {
-            const bool ok = seenA || mbar_wait(smem_addr(&fullA[u % R::RA]), (u / R::RA) & 1u, a.ctl);
+            const bool ok = seenA || mbar_wait_warp(smem_addr(&fullA[u % R::RA]), (u / R::RA) & 1u, a.ctl);
             seenA = false;
             return ok;
         };
         auto waitB = [&](unsigned u) {
-            const bool ok = seenB || mbar_wait(smem_addr(&fullB[u % R::RB]), (u / R::RB) & 1u, a.ctl);
+            const bool ok = seenB || mbar_wait_warp(smem_addr(&fullB[u % R::RB]), (u / R::RB) & 1u, a.ctl);
             seenB = false;
             return ok;
         };
-        auto lookA = [&](unsigned u) { seenA = mbar_test(smem_addr(&fullA[u % R::RA]), (u / R::RA) & 1u); };
-        auto lookB = [&](unsigned u) { seenB = mbar_test(smem_addr(&fullB[u % R::RB]), (u / R::RB) & 1u); };
-        for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x)
-            for (int c = 0; c < chunks && !s_abort; ++c, ++g_chunk) {
+        auto lookA = [&](unsigned u) { seenA = mbar_test_warp(smem_addr(&fullA[u % R::RA]), (u / R::RA) & 1u); };
+        auto lookB = [&](unsigned u) { seenB = mbar_test_warp(smem_addr(&fullB[u % R::RB]), (u / R::RB) & 1u); };
+        bool live = true;
+        for (int item = blockIdx.x; item < items && live; item += gridDim.x)
+            for (int c = 0; c < chunks; ++c, ++g_chunk) {
                 const unsigned buf = g_chunk & 1u, use = g_chunk >> 1;
-                if (use > 0 && !mbar_wait(smem_addr(&acce[buf]), (use - 1) & 1u, a.ctl)) { s_abort = 1; break; }
+                if (use > 0 && !mbar_wait_warp(smem_addr(&acce[buf]), (use - 1) & 1u, a.ctl)) { live = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t tacc = tmem + buf * (H * kT);
                 auto product = [&](unsigned u, unsigned v, int on) {
@@ -338,59 +340,59 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
                 for (; s < chunk; ++s) {
                     const int on = s > 0;
                     if constexpr (!SG) {
-                        if (!waitA(ua) || !waitB(ub)) { s_abort = 1; break; }
-                        lookB(ub + 1);
+                        if (!waitA(ua) || !waitB(ub)) break;
                         product(ua, ub, on);
                         mma_commit(smem_addr(&emptyB[ub % R::RB]));
-                        if (!waitB(ub + 1)) { s_abort = 1; break; }
-                        lookB(ub + 2);
+                        lookB(ub + 1);
+                        if (!waitB(ub + 1)) break;
                         product(ua, ub + 1, 1);
                         mma_commit(smem_addr(&emptyB[(ub + 1) % R::RB]));
-                        if (!waitB(ub + 2)) { s_abort = 1; break; }
-                        lookA(ua + 1);
-                        lookB(ub + 3);
+                        lookB(ub + 2);
+                        if (!waitB(ub + 2)) break;
                         product(ua, ub + 2, 1);
                         mma_commit(smem_addr(&emptyB[(ub + 2) % R::RB]));
                         mma_commit(smem_addr(&emptyA[ua % R::RA]));
+                        lookA(ua + 1);
+                        lookB(ub + 3);
                         ua += 1;
                         ub += 3;
                     } else {
-                        if (!waitA(ua) || !waitB(ub)) { s_abort = 1; break; }
-                        lookB(ub + 1);
+                        if (!waitA(ua) || !waitB(ub)) break;
                         product(ua, ub, on);
-                        if (!waitB(ub + 1)) { s_abort = 1; break; }
-                        lookA(ua + 1);
+                        lookB(ub + 1);
+                        if (!waitB(ub + 1)) break;
                         product(ua, ub + 1, 1);
                         mma_commit(smem_addr(&emptyA[ua % R::RA]));
                         mma_commit(smem_addr(&emptyB[(ub + 1) % R::RB]));
-                        if (!waitA(ua + 1)) { s_abort = 1; break; }
-                        lookA(ua + 2);
-                        lookB(ub + 2);
+                        lookA(ua + 1);
+                        if (!waitA(ua + 1)) break;
                         product(ua + 1, ub, 1);
                         mma_commit(smem_addr(&emptyA[(ua + 1) % R::RA]));
                         mma_commit(smem_addr(&emptyB[ub % R::RB]));
+                        lookA(ua + 2);
+                        lookB(ub + 2);
                         ua += 2;
                         ub += 2;
                     }
                 }
-                if (s < chunk) break;
+                if (s < chunk) { live = false; break; }
                 mma_commit(smem_addr(&accf[buf]));
             }
+        if (!live) s_abort = 1;
     } else if (warp >= 4) {
         const int quarter = warp & 3, half = (warp - 4) >> 2;
         unsigned g_chunk = 0;
-        for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+        bool ok = true;
+        for (int item = blockIdx.x; item < items; item += gridDim.x) {
             const int tm = item % a.tiles_m, tn = item / a.tiles_m;
             float acc[H][64];
 #pragma unroll
             for (int h = 0; h < H; ++h)
 #pragma unroll
                 for (int q = 0; q < 64; ++q) acc[h][q] = 0.0f;
-            bool ok = true;
             for (int c = 0; c < chunks; ++c, ++g_chunk) {
                 const unsigned buf = g_chunk & 1u, use = g_chunk >> 1;
-                ok = ok && mbar_wait(smem_addr(&accf[buf]), use & 1u, a.ctl);
-                __syncwarp();
+                ok = mbar_wait_warp(smem_addr(&accf[buf]), use & 1u, a.ctl);
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll
                 for (int h = 0; h < H; ++h)

@@ -97,7 +97,8 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
     unsigned long long my_spikes = 0;
     bool overflow = false;
 
-    for (int s = 0; s < a.steps && !s_abort; ++s) {
+    bool live = true;                              // no wait of this block has given up (the same for all threads)
+    for (int s = 0; s < a.steps; ++s) {
         const int t = a.t0 + s;
         const CUtensorMap *tmA = ((t + 1) & 1) ? &tmA1 : &tmA0;   // holds step t-1
         unsigned char *Aout = (t & 1) ? a.A1 : a.A0;
@@ -124,7 +125,7 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
                 for (int kb = 0; kb < kblocks; ++kb, ++g_mma) {
                     const int st = g_mma % kStages;
                     const unsigned round = g_mma / kStages;
-                    if (!mbar_wait(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
+                    if (!mbar_wait_warp(smem_addr(&full[st]), round & 1u, a.ctl)) { s_abort = 1; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const uint32_t dA = sbase + st * kStageBytes;
 #pragma unroll
@@ -158,10 +159,10 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
             __syncwarp();
             // epilogue: warps w, w+4, ... own TMEM lanes (tile rows) 32(w%4) ..,
             // each taking kEpiCols of the 128 columns
-            const bool ok = mbar_wait(smem_addr(&accbar), tiles_done & 1u, a.ctl);
+            if (!mbar_wait(smem_addr(&accbar), tiles_done & 1u, a.ctl)) s_abort = 1;
             ++tiles_done;
-            if (!ok) s_abort = 1;
             __syncthreads();                   // Poisson bits and parameters staged
+            live = !s_abort;                   // (nobody sets it before the tile's last barrier)
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const int b = m0 + bl;
             for (int cc = 0; cc < kEpiCols / 32; ++cc) {
@@ -172,7 +173,7 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
                 {
                     uint32_t v[32];
                     tmem_ld32(trow + (uint32_t)c0, v);
-                    if (!ok) continue;
+                    if (!live) continue;
                     const int j0 = n0 + c0;
                     // column q of this train at V[(j0 + q) * B + b], in groups of kSub
                     // columns whose loads are issued together
@@ -215,7 +216,7 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
                 my_spikes += (unsigned long long)__popc(bits);
             }
             __syncthreads();
-            if (ok) {
+            if (live) {
                 // spike bytes: 128-byte rows of A (the next step's operand);
                 // raster: the tile's four words of each train
                 for (int row = warp; row < kTM; row += kShThreads / 32)
@@ -229,13 +230,12 @@ shared_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ 
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncthreads();
-            if (s_abort) break;
+            if (!live) break;
         }
         // the spike bytes written this step are read by TMA (async proxy) next step
         asm volatile("fence.proxy.async.global;\n" ::: "memory");
         __syncthreads();
-        if (s_abort) break;
-        if (!grid_barrier(a.ctl)) { s_abort = 1; break; }
+        if (!live || !grid_barrier(a.ctl)) break;
         asm volatile("fence.proxy.async.global;\n" ::: "memory");
     }
 

@@ -184,7 +184,7 @@ shared_res_kernel(const __grid_constant__ CUtensorMap tmW, SharedArgs a) {
         }
         const unsigned long long key = a.pkey[row];
         const size_t part_words = (size_t)a.B * a.words;
-        for (int s = 0; s < a.steps && !s_abort; ++s) {
+        for (int s = 0; s < a.steps; ++s) {
             const int t = a.t0 + s;
             // words of step t - 1, stored by this launch with number s (or,
             // for its first step, prepared with number 0)
@@ -229,8 +229,8 @@ shared_res_kernel(const __grid_constant__ CUtensorMap tmW, SharedArgs a) {
                 // four draws a K block, while the MMAs of the others run
                 if (drawn < 32) draw4();
                 const unsigned round = ((unsigned)s * (unsigned)kblocks + (unsigned)i) / kStagesA;
-                if (ok && round > 0) ok = mbar_wait(smem_addr(&emptyA[part]), (round - 1) & 1u, a.ctl);
-                if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+                if (ok && round > 0) ok = mbar_wait_warp(smem_addr(&emptyA[part]), (round - 1) & 1u, a.ctl);
+                if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 tmem_st16(trow + kACol + (uint32_t)(part * 32), e[0]);
                 tmem_st16(trow + kACol + (uint32_t)(part * 32 + 16), e[1]);
@@ -242,8 +242,7 @@ shared_res_kernel(const __grid_constant__ CUtensorMap tmW, SharedArgs a) {
             }
             while (drawn < 32) draw4();
             if (!ok) { s_abort = 1; break; }
-            ok = mbar_wait(smem_addr(&accbar), (unsigned)s & 1u, a.ctl);
-            if (!__all_sync(0xffffffffu, ok)) { s_abort = 1; break; }
+            if (!mbar_wait_warp(smem_addr(&accbar), (unsigned)s & 1u, a.ctl)) { s_abort = 1; break; }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             unsigned bits = 0;
 #pragma unroll 1
@@ -296,26 +295,26 @@ shared_res_kernel(const __grid_constant__ CUtensorMap tmW, SharedArgs a) {
         for (unsigned i = issued > kStagesW ? issued - kStagesW : 0; i < issued; ++i)
             mbar_drain(smem_addr(&fullW[i % kStagesW]), (i / kStagesW) & 1u);
     } else if (warp == kOwners + 1) {
-        // MMAs; the next barriers are looked at before those at hand are issued
+        // MMAs; the next barriers are looked at while those at hand run
         constexpr uint32_t idesc = idesc_e4m3_f32(kTM, kTN);
         const uint64_t wdesc = umma_desc_sw128(sbase);
         bool ready = false;
-        for (int s = 0; s < a.steps && !s_abort; ++s) {
-            if (s > 0 && !mbar_wait(smem_addr(&accfree), (unsigned)(s - 1) & 1u, a.ctl)) { s_abort = 1; break; }
+        for (int s = 0; s < a.steps; ++s) {
+            if (s > 0 && !mbar_wait_warp(smem_addr(&accfree), (unsigned)(s - 1) & 1u, a.ctl)) { s_abort = 1; break; }
             int i = 0;
             for (; i < kblocks; ++i, ++issued) {
                 const unsigned sw = issued % kStagesW, sa = issued % kStagesA;
-                if (!ready && (!mbar_wait(smem_addr(&fullW[sw]), (issued / kStagesW) & 1u, a.ctl) ||
-                               !mbar_wait(smem_addr(&fullA[sa]), (issued / kStagesA) & 1u, a.ctl))) {
+                if (!ready && (!mbar_wait_warp(smem_addr(&fullW[sw]), (issued / kStagesW) & 1u, a.ctl) ||
+                               !mbar_wait_warp(smem_addr(&fullA[sa]), (issued / kStagesA) & 1u, a.ctl))) {
                     s_abort = 1;
                     break;
                 }
-                const unsigned nx = issued + 1;
-                ready = mbar_test(smem_addr(&fullW[nx % kStagesW]), (nx / kStagesW) & 1u) &&
-                        mbar_test(smem_addr(&fullA[nx % kStagesA]), (nx / kStagesA) & 1u);
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 mma_f8_block_ta(tmem, tmem + kACol + sa * 32, wdesc + sw * (kStageW / 16), idesc, i != 0,
                                 smem_addr(&emptyA[sa]), smem_addr(&emptyW[sw]));
+                const unsigned nx = issued + 1;
+                ready = __all_sync(0xffffffffu, mbar_test(smem_addr(&fullW[nx % kStagesW]), (nx / kStagesW) & 1u) &
+                                                    mbar_test(smem_addr(&fullA[nx % kStagesA]), (nx / kStagesA) & 1u));
             }
             if (i < kblocks) break;
             mma_commit(smem_addr(&accbar));

@@ -66,6 +66,31 @@ __device__ inline void mbar_drain(uint32_t bar, uint32_t parity) {
     }
 }
 
+// Both for a whole converged warp, with one answer for all its lanes.  Lanes that
+// poll for themselves may disagree around a timeout or another block's status, some
+// having seen the phase and others given up, and the warp-wide instructions that follow
+// (elections, TMEM loads and stores) need all of them.  The votes also keep what
+// follows uniform to the compiler: votes inside the polling loop, and a test behind the
+// MMAs instead of before them, cost nothing (shared_res_kernel 864 us a run with lanes
+// by themselves, 859 so, 974 with a vote after each lane's own wait).
+__device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_test(bar, parity));
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, Control *ctl) {
+    unsigned long long t0 = 0;
+    for (unsigned it = 0;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+        if ((it & 255u) == 255u) {
+            const unsigned long long now = global_timer_ns();
+            bool late = false;
+            if (t0 == 0) t0 = now;
+            else late = now - t0 > kWaitNs;
+            if (late) atomicCAS(&ctl->status, 0, (int)SN_ETIMEOUT);
+            if (__any_sync(0xffffffffu, late || ld_status(ctl) != 0)) return false;
+        }
+    }
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
