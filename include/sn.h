@@ -107,7 +107,8 @@ typedef enum {
 #define SN_PULL_PLAIN 0x1000u
 #define SN_PULL_CODED 0x2000u
                             /* sn_create only: the form of the pull store (see
-                               sn_pull_store_info).  Without either flag the
+                               sn_pull_store_info) for the kernel that takes
+                               one step at a time.  Without either flag the
                                library builds the plain form, ordered for
                                blocks of three steps; for a network of one
                                block of threads, or lists that form cannot

@@ -229,11 +229,11 @@ sn_status build_pull_store(sn_ctx *c) {
             byd[dstart[D - 1 - (int)(syn[p].x >> kPostBits)]++] = (uint32_t)p;
             pre_of[p] = (uint32_t)i;
         }
-    // The blocked kernel, unless the coded form is asked for, also where its
+    // The blocked kernel, unless a form is asked for, also where its
     // store outgrows the L2: it reads a synapse 0.44 times a step (10^5 neurons,
     // delays 1..16, 100 steps: 110 synapses a neuron 0.89 ms against 1.09 of
     // the best other form, 125: 1.04 against 1.22, 150 (147 MB): 1.19 against 1.50).
-    if (c->pull_hb && c->pin_format != 2) {
+    if (c->pull_hb && c->pin_format == 0) {
         const sn_status st = build_block_store(c, syn, byd, pre_of);
         if (st || c->pin_blocked) return st;
     }

@@ -1,0 +1,111 @@
+"""The pull store's forms on networks of many blocks: without a flag the order for
+blocks of three steps, SN_PULL_PLAIN and SN_PULL_CODED the kernel that takes one step
+at a time, and the same where the blocked kernel cannot count a list or hold a sum
+(a region of more than 131,070 synapses; integer weights whose magnitudes reach 2^31).
+Spikes and states equal the oracle's in every form."""
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2305_02510_gb300 import sn as S
+from paper_2305_02510_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+FORMS = [0, S.SN_PULL_PLAIN, S.SN_PULL_CODED]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__ as g
+    g.build()
+
+
+def plain_bytes(n, pre, post, delay, chunk):
+    """Bytes of the plain store in two regions (delay >= 2, delay 1), as the one-step
+    kernel reads it: within a block of `chunk` neurons by list length, then within 64
+    by the delay-1 list, pairs padded to the longest list of 32."""
+    long = np.bincount(post[delay >= 2], minlength=n)
+    one = np.bincount(post[delay == 1], minlength=n)
+    total = 0
+    for b0 in range(0, n, chunk):
+        order = b0 + np.argsort(-(long + one)[b0:b0 + chunk], kind="stable")
+        for w0 in range(0, order.size, 64):
+            part = order[w0:w0 + 64]
+            part = part[np.argsort(-one[part], kind="stable")]
+            for s0 in range(0, part.size, 32):
+                q = part[s0:s0 + 32]
+                total += ((int(long[q].max()) + 1) // 2 + (int(one[q].max()) + 1) // 2) * 32 * 16
+    return total
+
+
+def run(wl, form, steps):
+    ctx = S.from_workload(wl, flags=S.SN_PROP_PULL | form, record_steps=steps)
+    S.sn_run(ctx, steps)
+    raster = S.unpack_raster(S.sn_get_spikes(ctx, 0, steps), wl["n"])
+    v, r = S.sn_get_state(ctx)
+    return S.sn_pull_store_info(ctx), raster, np.asarray(v, np.float64), np.asarray(r)
+
+
+def check(wl, steps, mode, forms=FORMS):
+    st, want, _ = O.run(wl, mode, steps)
+    assert want.sum() > 100
+    info = []
+    for form in forms:
+        i, raster, v, r = run(wl, form, steps)
+        assert np.array_equal(raster, want) and np.array_equal(v, st.v) and np.array_equal(r, st.r), form
+        info.append(i)
+    return info
+
+
+@pytest.mark.parametrize("integer", [False, True])
+def test_flags_choose_the_kernel(integer):
+    n, steps = 3000, 60
+    wl = W.random_small(61, n=n, integer=integer, steps=steps, p=0.01, max_delay=9, events_rate=40.0)
+    auto, plain, coded = check(wl, steps, O.INT if integer else O.F32)
+    assert [i[0] for i in (auto, plain, coded)] == [S.SN_PULL_PLAIN, S.SN_PULL_PLAIN, S.SN_PULL_CODED]
+    pre, post, delay = (np.asarray(wl[k]) for k in ("pre", "post", "delay"))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    chunk = (-(-n // 32) + sms - 1) // sms * 32
+    assert plain[1] == plain_bytes(n, pre, post, delay, chunk) < auto[1]
+
+
+def test_a_list_too_long_to_count():
+    n, steps, m = 2000, 12, 131_072
+    rng = np.random.default_rng(8)
+    wl = W.random_small(62, n=n, integer=False, steps=steps, p=0.003, max_delay=5, events_rate=60.0)
+    order = np.argsort(np.concatenate([wl["pre"], pre := rng.integers(0, n, m)]), kind="stable")
+    add = dict(pre=pre, post=np.zeros(m), weight=rng.normal(0.0, 0.01, m), delay=np.full(m, 3))
+    for k, x in add.items():
+        wl[k] = np.concatenate([wl[k], x.astype(np.asarray(wl[k]).dtype)])[order]
+    auto, plain = check(wl, steps, O.F32, FORMS[:2])
+    assert auto == plain
+
+
+@pytest.mark.parametrize("together", [False, True])
+def test_integer_sums_past_32_bits(together):
+    """200 synapses of 16,000,000 into neuron 0: a sum of 3.2e9 leaves int32, a fifth
+    of it does not."""
+    n, steps, k = 2000, 10, 200
+    src = np.arange(100, 100 + k)
+    wl = W._base(n, "i32", np.where(np.arange(n) == 0, 2.0 ** 23, 5.0), np.zeros(n), np.zeros(n),
+                 np.zeros(n, np.int32), 4, steps)
+    wl.update(pre=src.astype(np.int32), post=np.zeros(k, np.int32), weight=np.full(k, 16e6),
+              delay=np.full(k, 4, np.int32), name="int-sums")
+    fire = src if together else src[:40]
+    wl["events"] = dict(step=np.repeat([1, 3, 4], fire.size).astype(np.int32),
+                        neuron=np.tile(fire, 3).astype(np.int32), value=np.full(3 * fire.size, 9.0))
+    if not together:
+        auto, plain, _ = check(wl, steps, O.INT)
+        assert auto == plain
+        return
+    for form in FORMS:
+        ctx = S.from_workload(wl, flags=S.SN_PROP_PULL | form, record_steps=steps)
+        S.sn_run(ctx, steps)
+        with pytest.raises(S.SnError) as e:
+            S.sn_sync(ctx)
+        assert e.value.status == S.SN_EOVERFLOW
