@@ -938,17 +938,21 @@ sn_status sn_run(sn_ctx *c, int32_t steps) {
         a.chunk = c->pull_chunk;
         a.j_first = c->shard_end ? c->shard_first : 0;
         a.j_end = c->shard_end ? c->shard_end : c->n;
-        e = c->pin_blocked ? launch_pull_block(a, c->dtype, c->pull_hb, c->pull_grid, c->pull_block_smem, c->stream)
+        const bool rows_live = c->ptag_live;
+        c->ptag_live = false;
+        e = c->pin_blocked ? launch_pull_block(a, c->dtype, c->pull_hb, c->pull_grid, c->pull_block_smem, rows_live,
+                                               c->stream)
                            : launch_sparse_pull(a, c->dtype, c->pin_coded != 0, c->pull_grid, c->pull_smem, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "simulation launch");
         c->hist_live = true;
+        c->ptag_live = c->pin_blocked;
     } else {
         if (c->kind == KIND_SPARSE && c->hist_live) {
             // spikes of a pull run whose deliveries are still due go to the ring
             if ((e = launch_pull_flush(a, c->dtype, (int)c->step, c->stream)) != cudaSuccess ||
                 (e = cudaMemsetAsync(c->hist, 0, (size_t)c->D * c->words * 4, c->stream)) != cudaSuccess)
                 return cuda_fail(c, e, "pull-to-push handover");
-            c->hist_live = false;
+            c->hist_live = c->ptag_live = false;
         }
         if (c->kind == KIND_SPARSE && !c->stdp && c->reg_grid > 0) {
             a.chunk = c->reg_chunk;
@@ -998,7 +1002,7 @@ sn_status sn_reset(sn_ctx *c) {
     if (c->spk) SN_CUDA(c, cudaMemsetAsync(c->spk, 0, (size_t)2 * c->words * 4, c->stream));
     if (c->trace) SN_CUDA(c, cudaMemsetAsync(c->trace, 0, 3 * vb, c->stream));
     if (c->hist) SN_CUDA(c, cudaMemsetAsync(c->hist, 0, (size_t)c->D * c->words * 4, c->stream));
-    c->hist_live = false;
+    c->hist_live = c->ptag_live = false;
     c->ring_live_until = 0;
     c->shard_known = 0;
     SN_CUDA(c, cudaMemsetAsync(c->raster, 0, (size_t)c->cap * c->words * 4, c->stream));
@@ -1120,6 +1124,7 @@ static sn_status rebuild_pending(sn_ctx *c) {
         sn_status s = dalloc(c, &c->hist, (size_t)D * row);
         if (s) return s;
     }
+    c->ptag_live = false;
     SN_CUDA(c, cudaMemsetAsync(c->hist, 0, (size_t)D * row, c->stream));
     for (long long tau = first; tau < t0; ++tau)
         SN_CUDA(c, cudaMemcpyAsync((char *)c->hist + (size_t)(tau % D) * row,
@@ -1322,6 +1327,7 @@ sn_status sn_load(sn_ctx *c, const void *buf, size_t size) {
         return cuda_fail(c, e, "load");
     }
     if (hd.has_trace && (e = put(c->trace, (size_t)3 * c->n * 4))) return cuda_fail(c, e, "load");
+    c->ptag_live = false;
     if (hd.has_hist) {
         if ((e = put(c->hist, (size_t)c->D * c->words * 4))) return cuda_fail(c, e, "load");
     } else if (c->hist) {

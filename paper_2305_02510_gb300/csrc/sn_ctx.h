@@ -50,6 +50,8 @@ struct sn_ctx {
     size_t pull_block_smem = 0;
     bool pin_blocked = false;          // the store is laid out for blocked pull (sn_pull_block.cu)
     unsigned long long *ptag = nullptr;
+    bool ptag_live = false;            // blocked pull: ptag holds the last rows of hist (the last run was one
+                                       // of its launches and nothing else has written hist since)
     bool pin_stale = true;             // the pull store must be (re)built from the CSR
     unsigned *hist = nullptr;          // [D][words] spike bits whose deliveries may be due
     bool hist_live = false;            // hist may hold spikes not yet delivered

@@ -253,7 +253,7 @@ cudaError_t launch_sparse_pull(const NetArgs &a, int dtype, bool coded, int grid
 cudaError_t plan_pull_block(int n, int D, int dtype, int grid, int chunk, int *hb, size_t *smem);
 size_t pull_tag_bytes(int words);
 unsigned pull_hist_byte(unsigned pre, int hb);
-cudaError_t launch_pull_block(NetArgs a, int dtype, int hb, int grid, size_t smem, cudaStream_t s);
+cudaError_t launch_pull_block(NetArgs a, int dtype, int hb, int grid, size_t smem, bool rows_live, cudaStream_t s);
 cudaError_t launch_pull_flush(const NetArgs &a, int dtype, int t0, cudaStream_t s);
 cudaError_t launch_gather_weights(const uint2 *syn, const long long *perm_inv, long long m,
                                   float *out, cudaStream_t s);

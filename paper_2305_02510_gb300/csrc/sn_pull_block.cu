@@ -36,7 +36,9 @@
 // That read is the only wait of a step (bounded, as the grid barrier's is);
 // everything that does not need the newest row (regions 0-3, the raster, the
 // external input of the next step) runs between the block's own store and
-// that read.  A row slot is reused after kTagRows steps; a block that has
+// that read.  Row t lies in slot t % kTagRows, so a launch that continues the last one
+// finds its rows in their slots; any other has them written from the history first.  A
+// row slot is reused after kTagRows steps; a block that has
 // read all of row t knows that every block has stored it, so no block is
 // more than one step ahead of another.
 //
@@ -298,7 +300,10 @@ __global__ void __launch_bounds__(MAXT, 1) pull_block_kernel(NetArgs a) {
         return w < W && tau >= 0 && tau >= t0 - D ? __ldcg(a.hist + (size_t)(tau % D) * W + w) : 0u;
     };
     if (threadIdx.x == 0) { s_stop = 0; s_fail = 0; }
-    for (int i = threadIdx.x; i < 2 * Wp; i += blockDim.x) s_rows[i] = 0u;
+    for (int i = threadIdx.x; i < Wp; i += blockDim.x) {
+        s_rows[((t0 - 3) & 1) * Wp + i] = hist_word(t0 - 3, i);
+        s_rows[(t0 & 1) * Wp + i] = hist_word(t0 - 2, i);
+    }
     if (use_h) {
         for (int i = threadIdx.x; i < (W + (W & 1)) * (HB / 4); i += blockDim.x) s_mem4[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
@@ -324,11 +329,20 @@ __global__ void __launch_bounds__(MAXT, 1) pull_block_kernel(NetArgs a) {
     // its block; n0..n2: of the next block's three steps
     Acc a0 = 0, a1 = 0, a2 = 0, n0 = 0, n1 = 0, n2 = 0;
     V ext = 0;                                          // external input of the step at hand
-    int k = 0;                                          // step within its block
+    int k = 2;                                          // step within its block
     int rslot = t0 % a.cap, hslot = t0 % D;             // raster and history rows of the step at hand
-    unit_load(ea, ent, 0, min(np(0), (hdr[0] + 1) >> 1));
-    // three steps before the first one only prepare its sums
-    for (int s = -3; s < a.steps; ++s) {
+    // the lists above delay 3 for a block of steps, from its words
+    auto three = [&](unsigned x, unsigned w) {
+        const unsigned bits = hist_bits<HB>(hist, x);
+        if (bits & 4u) n0 = BlockAcc<MODE>::add(n0, w);
+        if (bits & 2u) n1 = BlockAcc<MODE>::add(n1, w);
+        if (bits & 1u) n2 = BlockAcc<MODE>::add(n2, w);
+    };
+    // region 0 for the first block of steps; the rest of what comes before step 0
+    // is the last step of a block like any other's
+    unit_load(ea, ent, 0, np(0));
+    region_loop(ea, eb, ent, 0, np(0), hdr[0], 0, 0, three);
+    for (int s = -1; s < a.steps; ++s) {
         const int t = t0 + s;
         const unsigned char *row_prev = (const unsigned char *)(s_rows + ((t - 1) & 1) * Wp);   // step t - 1
         if (s >= 0) {
@@ -392,7 +406,7 @@ __global__ void __launch_bounds__(MAXT, 1) pull_block_kernel(NetArgs a) {
             }
             const unsigned ball = __ballot_sync(0xffffffffu, fire);
             if (word_lane) {
-                st_tagged(a.ptag + (size_t)(s & (kTagRows - 1)) * Wt + wword, (unsigned)s + 1u, ball);
+                st_tagged(a.ptag + (size_t)(t & (kTagRows - 1)) * Wt + wword, (unsigned)t + 1u, ball);
                 a.raster[(size_t)rslot * W + wword] = ball;
                 // the history's row of the step before: its slot held row t - 1 - D,
                 // which no block reads any more (every block has stored row t - 1)
@@ -419,7 +433,7 @@ __global__ void __launch_bounds__(MAXT, 1) pull_block_kernel(NetArgs a) {
             // the thread's columns of row t - 3 enter the words below, the first
             // pair loaded ahead (its slot is stored again only at step t + 5,
             // when every block has passed here)
-            const unsigned long long *tag3 = a.ptag + (size_t)((s - 3) & (kTagRows - 1)) * Wt;
+            const unsigned long long *tag3 = a.ptag + (size_t)((t - 3) & (kTagRows - 1)) * Wt;
             auto oldest = [&](int i) -> uint2 {
                 if (2 * i >= W) return make_uint2(0u, 0u);
                 const ulonglong2 x = ld_tagged2(tag3 + 2 * i);
@@ -429,7 +443,7 @@ __global__ void __launch_bounds__(MAXT, 1) pull_block_kernel(NetArgs a) {
             if (k == 2 && use_h) old = oldest(threadIdx.x);
             // external input of the next step
             ext = 0;
-            if (mine && s >= -1) {
+            if (mine) {
                 const int tn = t + 1;
                 if (tn < a.ev_nsteps) {
                     int lo = a.ev_off[tn], hi = a.ev_off[tn + 1];
@@ -459,13 +473,7 @@ __global__ void __launch_bounds__(MAXT, 1) pull_block_kernel(NetArgs a) {
             }
             if (k == 2) unit_load(ea, ent + (size_t)atA * 32, 0, npA);
             // delays above 3 of the next block's steps
-            region_loop(ea, eb, ent, atA, npA, npAmax, k == 1 ? hdr[6] : hdr[5], k == 1 ? np(3) : np(2),
-                        [&](unsigned x, unsigned w) {
-                            const unsigned bits = hist_bits<HB>(hist, x);
-                            if (bits & 4u) n0 = BlockAcc<MODE>::add(n0, w);
-                            if (bits & 2u) n1 = BlockAcc<MODE>::add(n1, w);
-                            if (bits & 1u) n2 = BlockAcc<MODE>::add(n2, w);
-                        });
+            region_loop(ea, eb, ent, atA, npA, npAmax, k == 1 ? hdr[6] : hdr[5], k == 1 ? np(3) : np(2), three);
             if (k == 2) {
                 // delay 3 of the next block's first two steps: rows t - 2, t - 1
                 region_loop(ea, eb, ent, hdr[5], np(2), hdr[2], hdr[6], np(3), [&](unsigned x, unsigned w) {
@@ -483,20 +491,18 @@ __global__ void __launch_bounds__(MAXT, 1) pull_block_kernel(NetArgs a) {
                     });
             }
             // delay 2 of the next step: row t - 1
-            region_loop(ea, eb, ent, hdr[6], np(3), hdr[3], s >= -1 ? hdr[7] : halfA,
-                        s >= -1 ? np(4) : max(np(0) - halfA, 0), [&](unsigned x, unsigned w) {
-                            if (row_bit(row_prev, x)) a0 = BlockAcc<MODE>::add(a0, w);
-                        });
+            region_loop(ea, eb, ent, hdr[6], np(3), hdr[3], hdr[7], np(4), [&](unsigned x, unsigned w) {
+                if (row_bit(row_prev, x)) a0 = BlockAcc<MODE>::add(a0, w);
+            });
         }
         // ---- the row of step t, in place of row t - 2 (read in this phase
         // only when it ends a block)
         unsigned *row = s_rows + (t & 1) * Wp;
         if (k == 2) __syncthreads();
         if (s >= 0) {
-            if (!read_row(a.ptag + (size_t)(s & (kTagRows - 1)) * Wt, W, (unsigned)s + 1u, row, a.ctl)) s_fail = 1;
+            if (!read_row(a.ptag + (size_t)(t & (kTagRows - 1)) * Wt, W, (unsigned)t + 1u, row, a.ctl)) s_fail = 1;
         } else {
-            const unsigned long long *src = a.ptag + (size_t)(s & (kTagRows - 1)) * Wt;
-            for (int i = threadIdx.x; i < W; i += blockDim.x) row[i] = (unsigned)__ldcg(src + i);
+            for (int i = threadIdx.x; i < W; i += blockDim.x) row[i] = hist_word(t, i);
         }
         k = k == 2 ? 0 : k + 1;
         if (threadIdx.x == 0) s_stop = st;
@@ -525,14 +531,15 @@ __global__ void __launch_bounds__(MAXT, 1) pull_block_kernel(NetArgs a) {
 }
 
 
-// The tagged slots at the start of a launch: slot q holds row t0 - kTagRows + q
-// of the history with step number 0 (a launch's own steps count from 1).
-__global__ void pull_tag_init_kernel(NetArgs a) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kTagRows * a.wt) return;
-    const int tau = a.t0 - kTagRows + i / a.wt, w = i % a.wt;
+// The rows of the last kTagRows steps from the history into their slots (all of them:
+// no number of a later step is left behind).
+__global__ void pull_rows_kernel(NetArgs a) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, q = i / a.wt, w = i % a.wt;
+    if (q >= kTagRows) return;
+    const int tau = a.t0 - kTagRows + q;
     const bool in = tau >= 0 && tau >= a.t0 - a.hD && w < a.words;
-    a.ptag[i] = in ? a.hist[(size_t)(tau % a.hD) * a.words + w] : 0u;
+    a.ptag[(size_t)(tau & (kTagRows - 1)) * a.wt + w] =
+        (unsigned long long)((unsigned)tau + 1u) << 32 | (in ? a.hist[(size_t)(tau % a.hD) * a.words + w] : 0u);
 }
 
 template <int HB, int MAXT>
@@ -587,17 +594,24 @@ unsigned pull_hist_byte(unsigned pre, int hb) {
     return (pair * 2 * hb + piece_slot((int)pair, (int)l, hb) * v + jj % v) * 4u + (jj / v) * (hb / 8);
 }
 
-cudaError_t launch_pull_block(NetArgs a, int dtype, int hb, int grid, size_t smem, cudaStream_t s) {
+// rows_live: the slots hold the last rows (the last launch of this kernel ended at
+// step t0, and nothing has changed the history since).
+cudaError_t launch_pull_block(NetArgs a, int dtype, int hb, int grid, size_t smem, bool rows_live, cudaStream_t s) {
     a.wp = (a.words + 3) & ~3;
     a.wt = (a.words + 1) & ~1;
     a.rows_at = a.hD > 3 ? a.wt * hb * 4 : 0;
     a.acc_at = a.rows_at + 2 * a.wp * 4;
     void *args[] = {(void *)&a};
     const void *fn = block_fn(dtype, hb, a.chunk);
-    const int total = kTagRows * a.wt;
-    pull_tag_init_kernel<<<(total + 255) / 256, 256, 0, s>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &capture);
     if (e != cudaSuccess) return e;
+    // (a graph may be launched again after something else has run)
+    if (!rows_live || capture != cudaStreamCaptureStatusNone) {
+        const int total = kTagRows * a.wt;
+        pull_rows_kernel<<<(total + 255) / 256, 256, 0, s>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     // cooperative: the blocks wait for one another's rows, so all must be resident
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(a.chunk), args, smem, s);
 }

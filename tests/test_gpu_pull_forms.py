@@ -109,3 +109,74 @@ def test_integer_sums_past_32_bits(together):
         with pytest.raises(S.SnError) as e:
             S.sn_sync(ctx)
         assert e.value.status == S.SN_EOVERFLOW
+
+
+def drive(form, n, max_delay, integer):
+    """Runs of one and a few steps, a reset after fewer and after more steps than there
+    are row slots, a checkpoint taken back, weights replaced with spikes in flight, a
+    push run in between: every raster and state along the way."""
+    wl = W.random_small(63, n=n, integer=integer, steps=60, p=12.0 / n, max_delay=max_delay, events_rate=n / 60.0)
+    ctx = S.from_workload(wl, flags=S.SN_PROP_PULL | form, record_steps=60)
+    out = []
+
+    def look(t0, t1):
+        out.append(S.sn_get_spikes(ctx, t0, t1).copy())
+        out.extend(np.asarray(x).copy() for x in S.sn_get_state(ctx))
+
+    for runs in ((1, 1, 1), (5,), (1,) * 12 + (2, 3, 7, 1, 1), (30,)):
+        S.sn_reset(ctx)
+        for q in runs:
+            S.sn_run(ctx, q)
+        look(0, sum(runs))
+    if not integer:
+        S.sn_set_weights(ctx, np.asarray(wl["weight"], np.float32)[::-1].copy())
+    S.sn_run(ctx, 4)
+    look(30, 34)
+    blob = S.sn_save(ctx)
+    S.sn_run(ctx, 6)
+    look(34, 40)
+    S.sn_load(ctx, blob)
+    S.sn_run(ctx, 1)
+    S.sn_run(ctx, 5)
+    look(34, 40)
+    for mode, q in ((S.SN_PUSH, 3), (S.SN_PULL, 1), (S.SN_PULL, 4), (S.SN_PUSH, 1), (S.SN_PULL, 6)):
+        S.sn_set_propagation(ctx, mode)
+        S.sn_run(ctx, q)
+    look(40, 55)
+    return out
+
+
+@pytest.mark.parametrize("integer", [False, True])
+@pytest.mark.parametrize("n,max_delay", [(1100, 1), (2500, 3), (2500, 4), (2500, 16), (40_001, 9)])
+def test_rows_between_launches(n, max_delay, integer):
+    want = drive(S.SN_PULL_PLAIN, n, max_delay, integer)
+    assert sum(int(S.unpack_raster(w, n).sum()) for w in want[9:10]) > 100
+    for k, (a, b) in enumerate(zip(drive(0, n, max_delay, integer), want)):
+        assert np.array_equal(a, b), k
+
+
+def test_captured_run_after_a_reset():
+    """A captured run of 20 steps from step 0, launched again after a reset and other
+    runs, gives the same steps."""
+    wl = W.random_small(64, n=2500, integer=True, steps=20, p=0.005, max_delay=16, events_rate=40.0)
+    stream = torch.cuda.Stream()
+    ctx = S.from_workload(wl, flags=S.SN_PROP_PULL, record_steps=20, stream=stream.cuda_stream)
+    S.sn_run(ctx, 20)
+    S.sn_sync(ctx)
+    want = S.sn_get_spikes(ctx, 0, 20).copy()
+    v = np.asarray(S.sn_get_state(ctx)[0]).copy()
+    assert S.unpack_raster(want, 2500).sum() > 100
+    S.sn_reset(ctx)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        S.sn_run(ctx, 20)
+    for runs in ((), (1, 1, 1), (20,)):
+        S.sn_reset(ctx)
+        for q in runs:
+            S.sn_run(ctx, q)
+        S.sn_reset(ctx)
+        with torch.cuda.stream(stream):
+            graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(np.asarray(S.sn_get_state(ctx)[0]), v)
