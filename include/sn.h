@@ -110,11 +110,12 @@ typedef enum {
                                sn_pull_store_info) for the kernel that takes
                                one step at a time.  Without either flag the
                                library builds the plain form, ordered for
-                               blocks of three steps; for a network of one
-                               block of threads, or lists that form cannot
-                               count, the plain form while it takes at most
-                               80 % of the L2 cache, else the smaller form.
-                               The forms
+                               blocks of three steps, where that kernel is the
+                               faster one; for a network of one block of
+                               threads, for lists it cannot count, and for
+                               short delays in large stores, the plain form
+                               while it takes at most 80 % of the L2 cache,
+                               else the smaller form.  The forms
                                hold the same synapses in the same order, so
                                the results are identical; the flags let tests
                                and tuning run either                          */

@@ -103,77 +103,121 @@ sn_status upload_pull_store(sn_ctx *c, const std::vector<uint4> &pin, const std:
     return SN_OK;
 }
 
-// The store of the blocked kernel (sn_pull_block.cu), from the CSR positions
-// `byd` in list order: five regions by delay per slice of 32 positions, each
-// padded to the slice's longest list.  Within each block's neurons the lists
-// are sorted by the first region (the longest work), then within runs of
-// three warps by the delay-1 region (on the step's critical path, and walked
-// three times as often).  Not built (pin_blocked stays false) for lists the
-// kernel cannot count or sum.
-sn_status build_block_store(sn_ctx *c, const std::vector<uint2> &syn, const std::vector<uint32_t> &byd,
-                            const std::vector<uint32_t> &pre_of) {
-    constexpr int kRegions = 5;
-    const int n = c->n, hb = c->pull_hb, slices = (n + 31) / 32;
+constexpr int kPullRegions = 5;
+
+// Region of a synapse of delay d in the blocked kernel's store.
+int pull_region(int d) { return d >= 7 ? 0 : d >= 4 ? 1 : 5 - d; }
+
+// Layout of the blocked kernel's store (sn_pull_block.cu): five regions by delay per
+// slice of 32 positions, each padded to the slice's longest list.  Within each
+// block's neurons the lists are sorted by the first region (the longest work), then
+// within runs of three warps by the delay-1 region (on the step's critical path, and
+// walked three times as often).
+struct BlockPlan {
+    bool ok = false;                       // the kernel can count every list and hold every sum
+    std::vector<int> perm, lens;           // neuron of each position; [regions][n] entries by position
+    std::vector<long long> off, start;     // first uint4 of each slice, and [regions][slices] of its regions
+    long long total = 0;                   // uint4s of the store
+    double reads = 0;                      // and those a step reads: a third of the regions above delay 3,
+                                           // two of delay 3's for three steps, the others whole
+};
+
+BlockPlan plan_block_store(const sn_ctx *c, const std::vector<uint2> &syn) {
+    const int n = c->n, slices = (n + 31) / 32;
     const long long m = c->m;
-    c->pin_blocked = false;
-    auto region_of = [&](uint32_t p) {
-        const int d = (int)(syn[p].x >> kPostBits) + 1;
-        return d >= 7 ? 0 : d >= 4 ? 1 : 5 - d;
-    };
-    std::vector<int> len(kRegions * (size_t)n, 0);
-    for (long long k = 0; k < m; ++k) len[(size_t)region_of(byd[k]) * n + (syn[byd[k]].x & kPostMask)]++;
+    BlockPlan p;
+    std::vector<int> len(kPullRegions * (size_t)n, 0);
+    for (long long k = 0; k < m; ++k)
+        len[(size_t)pull_region((int)(syn[k].x >> kPostBits) + 1) * n + (syn[k].x & kPostMask)]++;
     // the kernel counts a region's pairs in 16 bits and sums integers in 32
     for (const int q : len)
-        if (q > 2 * 65535) return SN_OK;
+        if (q > 2 * 65535) return p;
     if (c->dtype == SN_I32) {
         std::vector<long long> sum(n, 0);
         for (long long k = 0; k < m; ++k) sum[syn[k].x & kPostMask] += std::llabs((long long)(int)syn[k].y);
         for (const long long q : sum)
-            if (q > 2147483647ll) return SN_OK;
+            if (q > 2147483647ll) return p;
     }
-    std::vector<int> perm(n), pos_of(n);
-    for (int j = 0; j < n; ++j) perm[j] = j;
+    p.perm.resize(n);
+    for (int j = 0; j < n; ++j) p.perm[j] = j;
     auto by_region = [&](int r) {
         return [&len, n, r](int x, int y) { return len[(size_t)r * n + x] > len[(size_t)r * n + y]; };
     };
     for (int b0 = 0; b0 < n; b0 += c->pull_chunk) {
         const int b1 = std::min(n, b0 + c->pull_chunk);
-        std::stable_sort(perm.begin() + b0, perm.begin() + b1, by_region(0));
+        std::stable_sort(p.perm.begin() + b0, p.perm.begin() + b1, by_region(0));
         for (int w0 = b0; w0 < b1; w0 += 96)
-            std::stable_sort(perm.begin() + w0, perm.begin() + std::min(b1, w0 + 96), by_region(4));
+            std::stable_sort(p.perm.begin() + w0, p.perm.begin() + std::min(b1, w0 + 96), by_region(4));
     }
-    for (int q = 0; q < n; ++q) pos_of[perm[q]] = q;
-    std::vector<long long> off(slices), start(kRegions * (size_t)slices);
-    std::vector<int> lens(kRegions * (size_t)n);
-    long long total = 0;
+    p.off.resize(slices);
+    p.start.resize(kPullRegions * (size_t)slices);
+    p.lens.resize(kPullRegions * (size_t)n);
+    const double per_step[kPullRegions] = {1.0 / 3, 1.0 / 3, 2.0 / 3, 1.0, 1.0};
     for (int sl = 0; sl < slices; ++sl) {
-        off[sl] = total;
-        for (int r = 0; r < kRegions; ++r) {
+        p.off[sl] = p.total;
+        for (int r = 0; r < kPullRegions; ++r) {
             int longest = 0;
             for (int q = sl * 32; q < std::min(n, sl * 32 + 32); ++q) {
-                lens[(size_t)r * n + q] = len[(size_t)r * n + perm[q]];
-                longest = std::max(longest, lens[(size_t)r * n + q]);
+                p.lens[(size_t)r * n + q] = len[(size_t)r * n + p.perm[q]];
+                longest = std::max(longest, p.lens[(size_t)r * n + q]);
             }
-            start[(size_t)r * slices + sl] = total;
-            total += (long long)((longest + 1) / 2) * 32;
+            const long long units = (long long)((longest + 1) / 2) * 32;
+            p.start[(size_t)r * slices + sl] = p.total;
+            p.total += units;
+            p.reads += per_step[r] * (double)units;
         }
     }
-    std::vector<uint4> pin(std::max(total, 1ll), make_uint4(0, 0, 0, 0));
-    std::fill(len.begin(), len.end(), 0);                // entries placed so far
+    p.ok = true;
+    return p;
+}
+
+// Whether the blocked kernel is the faster one, beside the one-step kernel over a
+// store of `old` bytes (or at least as many; old_coded: in the coded form).  Both
+// sides measured, float, 200 steps, us a step, the one-step kernel second; r is the
+// bytes that a step reads in proportion to the other store's.
+//  - Narrow blocks (up to 102,144 neurons on 152 SMs): a store well inside the L2, at
+//    any delays: from 2.3 | 3.6 (3000 x 30, delay 1) to 8.4 | 8.2 (100,000 x 80, delays
+//    1, 2).  Beyond that where r <= 1: 100,000 x 100 delays 1, 2 (98 MB, r 1.07) 10.9 |
+//    9.5, delays 1..3 (1.02) 9.7 | 9.6, 1..4 (0.91) 9.8 | 9.6, 1..6 (0.78) 9.0 | 9.7;
+//    125 delays 1..4 (1.14) 12.7 | 11.7, 1..6 (0.97) 11.5 | 11.6, 1..16 (0.71) 9.9 | 12.0;
+//    150 delay 1 (1.38) 22.7 | 12.8.  Where the other store does not stay in the L2 either,
+//    r <= 1.2: 200 delays 1..4 (1.12) 22.1 | 25.0, 1..3 (1.28) 26.2 | 25.7.
+//  - Wide blocks walk slower (64 registers, spills, units of two loads): small stores
+//    (110,000 x 10, delays 1..3, 3.6 | 4.3), delay 1 alone up to a third of the L2
+//    (110,000 x 45 6.6 | 6.8; 140,000 x 60 9.4 | 9.1), and r <= 0.78: 110,000 x 60
+//    delays 1..8 (0.75) 7.2 | 7.3, 1..12 (0.66) 6.8 | 7.9, 140,000 x 30 delays 1..10
+//    (0.77) 6.2 | 6.7, 1..8 (0.84) 6.5 | 6.4, 1..3 (1.14) 6.7 | 6.3.  Not past the L2
+//    beside a plain store within it: 110,000 x 100 delays 1..12 (0.61) 11.3 | 10.4.
+bool block_store_wins(const sn_ctx *c, const BlockPlan &p, double l2, double old, bool old_coded) {
+    const double bytes = (double)p.total * 16.0, reads = p.reads * 16.0;
+    if (c->pull_chunk <= kPullNarrow) return bytes <= 0.72 * l2 || reads <= (old <= 0.8 * l2 ? 1.0 : 1.2) * old;
+    return bytes <= 0.16 * l2 || (c->D == 1 && bytes <= 0.35 * l2) ||
+           (reads <= 0.78 * old && (old_coded || bytes <= 0.85 * l2));
+}
+
+// The store of the blocked kernel, from the CSR positions `byd` in list order.
+sn_status build_block_store(sn_ctx *c, const BlockPlan &plan, const std::vector<uint2> &syn,
+                            const std::vector<uint32_t> &byd, const std::vector<uint32_t> &pre_of) {
+    const int n = c->n, slices = (n + 31) / 32;
+    const long long m = c->m;
+    std::vector<int> pos_of(n);
+    for (int q = 0; q < n; ++q) pos_of[plan.perm[q]] = q;
+    std::vector<uint4> pin(std::max(plan.total, 1ll), make_uint4(0, 0, 0, 0));
+    std::vector<int> len(kPullRegions * (size_t)n, 0);   // entries placed so far
     std::vector<unsigned> word_at(n);
-    for (int i = 0; i < n; ++i) word_at[i] = pull_hist_byte((unsigned)i, hb) << 5;
+    for (int i = 0; i < n; ++i) word_at[i] = pull_hist_byte((unsigned)i, c->pull_hb) << 5;
     for (long long k = 0; k < m; ++k) {
         const uint32_t p = byd[k], pre = pre_of[p];
-        const int d = (int)(syn[p].x >> kPostBits) + 1, r = region_of(p), j = (int)(syn[p].x & kPostMask);
+        const int d = (int)(syn[p].x >> kPostBits) + 1, r = pull_region(d), j = (int)(syn[p].x & kPostMask);
         const int ps = pos_of[j], q = len[(size_t)r * n + j]++;
         const unsigned x = r == 0 ? word_at[pre] | (unsigned)(d - 7)
                          : r == 1 ? word_at[pre] | (unsigned)(d - 4) : (pre >> 5) << 7 | (pre & 31u);
-        uint4 &u = pin[start[(size_t)r * slices + (ps >> 5)] + (long long)(q >> 1) * 32 + (ps & 31)];
+        uint4 &u = pin[plan.start[(size_t)r * slices + (ps >> 5)] + (long long)(q >> 1) * 32 + (ps & 31)];
         if (q & 1) { u.z = x; u.w = syn[p].y; } else { u.x = x; u.y = syn[p].y; }
     }
     sn_status s;
     if (!c->ptag && (s = dalloc(c, &c->ptag, pull_tag_bytes(c->words)))) return s;
-    if ((s = upload_pull_store(c, pin, off, lens, perm))) return s;
+    if ((s = upload_pull_store(c, pin, plan.off, plan.lens, plan.perm))) return s;
     c->pin_coded = 0;
     c->pin_blocked = true;
     c->pin_entries = m;
@@ -183,7 +227,8 @@ sn_status build_block_store(sn_ctx *c, const std::vector<uint2> &syn, const std:
 
 // Incoming synapses of every neuron in the canonical order of the float sum:
 // descending delay, then ascending pre and input index (the oldest spikes
-// first), laid out for the pull kernel in two regions per slice of 32 neurons
+// first).  The blocked kernel's store where it is the faster one (block_store_wins),
+// else laid out for the one-step kernel in two regions per slice of 32 neurons
 // (neurons 32s .. 32s+31): first the synapses of delay >= 2 (the ones a step
 // can add before the previous step's spikes are in), then those of delay 1.
 // A synapse's bit in the kernel's spike window lies y = (D - d) * Wp * 32 + pre
@@ -229,14 +274,17 @@ sn_status build_pull_store(sn_ctx *c) {
             byd[dstart[D - 1 - (int)(syn[p].x >> kPostBits)]++] = (uint32_t)p;
             pre_of[p] = (uint32_t)i;
         }
-    // The blocked kernel, unless a form is asked for, also where its
-    // store outgrows the L2: it reads a synapse 0.44 times a step (10^5 neurons,
-    // delays 1..16, 100 steps: 110 synapses a neuron 0.89 ms against 1.09 of
-    // the best other form, 125: 1.04 against 1.22, 150 (147 MB): 1.19 against 1.50).
-    if (c->pull_hb && c->pin_format == 0) {
-        const sn_status st = build_block_store(c, syn, byd, pre_of);
-        if (st || c->pin_blocked) return st;
-    }
+    int l2 = 0, dev = 0;
+    SN_CUDA(c, cudaGetDevice(&dev));
+    SN_CUDA(c, cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+    // the blocked kernel where it is the faster one, unless a form is asked for (no
+    // other form takes less than 6 bytes a synapse; its size is only worked out where
+    // that does not settle it)
+    c->pin_blocked = false;
+    BlockPlan plan;
+    if (c->pull_hb && c->pin_format == 0) plan = plan_block_store(c, syn);
+    if (plan.ok && block_store_wins(c, plan, l2, 6.0 * (double)m, false))
+        return build_block_store(c, plan, syn, byd, pre_of);
     const bool one_region = c->pull_grid == 1;
     const unsigned long long wbits = (unsigned long long)((c->words + 3) & ~3) * 32;   // window row, bits
     auto region_of = [&](uint32_t p) { return ((syn[p].x >> kPostBits) == 0 && !one_region) ? 1 : 0; };
@@ -300,11 +348,10 @@ sn_status build_pull_store(sn_ctx *c) {
     // the library's choice: the plain form (fewer instructions a synapse)
     // while its store stays well inside the L2, which serves it every step;
     // the coded form when that keeps the store smaller
-    int l2 = 0, dev = 0;
-    SN_CUDA(c, cudaGetDevice(&dev));
-    SN_CUDA(c, cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
     const bool plain_fits = (double)total[0] * 16 <= 0.8 * (double)l2;
     const int f = c->pin_format == 1 ? 0 : c->pin_format == 2 ? 1 : (!plain_fits && total[1] < total[0] ? 1 : 0);
+    if (plan.ok && block_store_wins(c, plan, l2, (double)total[f] * 16, f == 1))
+        return build_block_store(c, plan, syn, byd, pre_of);
     const long long tot = std::max(total[f], 1ll);
     std::vector<uint4> pin(tot, make_uint4(0, 0, 0, 0));
     auto comp = [](uint4 &v, int i) -> unsigned & { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; };
@@ -349,7 +396,6 @@ sn_status build_pull_store(sn_ctx *c) {
     if (s) return s;
     SN_CUDA(c, cudaMemcpy(c->pin_y0, y0p.data(), (size_t)n * 8, cudaMemcpyHostToDevice));
     c->pin_coded = f;
-    c->pin_blocked = false;
     c->pin_entries = 0;
     for (const int q : lens) c->pin_entries += q;
     c->pin_stale = false;

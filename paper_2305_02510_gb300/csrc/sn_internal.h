@@ -249,7 +249,9 @@ cudaError_t plan_pull(int n, int D, long long m, int *grid, int *chunk, int *row
 cudaError_t launch_shard_put(unsigned *hist, unsigned *raster, int D, int cap, int words, int w0, int w1,
                              long long t0, int rows, const unsigned *src, cudaStream_t s);
 cudaError_t launch_sparse_pull(const NetArgs &a, int dtype, bool coded, int grid, size_t smem, cudaStream_t s);
-// Pull in blocks of three steps (sn_pull_block.cu).
+// Pull in blocks of three steps (sn_pull_block.cu).  Blocks of up to kPullNarrow threads
+// have 80 registers a thread, wider ones 64.
+constexpr int kPullNarrow = 672;
 cudaError_t plan_pull_block(int n, int D, int dtype, int grid, int chunk, int *hb, size_t *smem);
 size_t pull_tag_bytes(int words);
 unsigned pull_hist_byte(unsigned pre, int hb);

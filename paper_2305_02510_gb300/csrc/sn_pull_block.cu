@@ -72,12 +72,12 @@ template <> struct BlockAcc<SN_I32> {
 };
 
 constexpr int kTagRows = 8;         // slots of the tagged spike rows (at least 5: see the kernel)
-// Blocks of up to kBlkThreads threads have 80 registers a thread, wider ones 64;
+// Blocks of up to kPullNarrow threads have 80 registers a thread, wider ones 64;
 // a unit (half of the double buffer) is 3 or 2 16-byte loads of two synapses
-// each.  No instantiation may spill: next to 228 KB of shared memory the L1 is
-// too small, and 50 bytes of spills a thread cost 15 % of the step.
-constexpr int kBlkThreads = 672;
-template <int MAXT> constexpr int unit_of() { return MAXT <= kBlkThreads ? 3 : 2; }
+// each.  The narrow form may not spill: next to 228 KB of shared memory the L1 is
+// too small, and 50 bytes of spills a thread cost 15 % of the step.  The wide one
+// spills up to 40 bytes, and the host takes it by a stricter rule (block_store_wins).
+template <int MAXT> constexpr int unit_of() { return MAXT <= kPullNarrow ? 3 : 2; }
 
 constexpr int kCols = 3;            // 16-byte reads of a row a thread has in flight: words / 2 <= kCols * threads
 
@@ -549,11 +549,11 @@ const void *block_fn_of(int dtype) {
 }
 
 const void *block_fn(int dtype, int hb, int threads) {
-    const bool wide = threads > kBlkThreads;
+    const bool wide = threads > kPullNarrow;
     switch (hb) {
-        case 8: return wide ? block_fn_of<8, kPullMaxBlock>(dtype) : block_fn_of<8, kBlkThreads>(dtype);
-        case 16: return wide ? block_fn_of<16, kPullMaxBlock>(dtype) : block_fn_of<16, kBlkThreads>(dtype);
-        default: return wide ? block_fn_of<32, kPullMaxBlock>(dtype) : block_fn_of<32, kBlkThreads>(dtype);
+        case 8: return wide ? block_fn_of<8, kPullMaxBlock>(dtype) : block_fn_of<8, kPullNarrow>(dtype);
+        case 16: return wide ? block_fn_of<16, kPullMaxBlock>(dtype) : block_fn_of<16, kPullNarrow>(dtype);
+        default: return wide ? block_fn_of<32, kPullMaxBlock>(dtype) : block_fn_of<32, kPullNarrow>(dtype);
     }
 }
 
