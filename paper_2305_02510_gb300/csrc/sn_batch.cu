@@ -183,7 +183,7 @@ __device__ __forceinline__ void add_shared(unsigned long long *p, unsigned long 
 }
 __device__ __forceinline__ void add_shared(unsigned *p, unsigned x) { atomicAdd(p, x); }
 
-// All steps of a network of at most kOwn * LANES neurons, by a block (LANES =
+// All steps of a network of at most SLOTS * LANES neurons, by a block (LANES =
 // 256) or a warp (32).  A step of the general form below is five dependent
 // trips to memory: state and parameters, event range, row bounds, synapses, and
 // the stores in between.  Here a thread keeps the state and the parameters of its
@@ -191,14 +191,17 @@ __device__ __forceinline__ void add_shared(unsigned *p, unsigned x) { atomicAdd(
 // input of t + 1 is prepared while the first synapses of step t are on their way:
 // one trip a step, 4.6 -> 2.5 us at 1021 neurons with two blocks an SM.  What bounds it now is the instruction
 // issue of an SM's 16 warps (the draws' 64-bit multiplies, the rule, the synapses).
-// `list` holds kOwn * LANES rows and `rows` as many; `cnt` two counters, both
+// A network of one neuron a thread at most takes SLOTS = 1: the rule and the draws of
+// three empty slots made 2000 of 130 neurons 9 % slower than the general form (885 ->
+// 961 us, 523 with one slot).
+// `list` holds SLOTS * LANES rows and `rows` as many; `cnt` two counters, both
 // zero.  (The row bounds lie in shared memory and the amplitudes, which few
 // neurons need in a step, in global: at 128 registers a thread anything more
 // spills, and with 28 KB of L1 left a spill is a trip to L2.)
 constexpr int kOwn = 4;
 static_assert(kListInts >= 4 * kOwn * kBatchBlock, "rows and list of a block (and of its warps)");
 
-template <int MODE, int LANES>
+template <int MODE, int LANES, int SLOTS>
 __device__ __forceinline__ void run_own(const BatchArgs &a, const BatchNet<MODE> &nb, typename Tr<MODE>::A *ring,
                                         bool global_ring, int tid, int2 *list, int2 *rows, int *cnt,
                                         unsigned long long &my_spikes, unsigned long long &my_events,
@@ -207,14 +210,14 @@ __device__ __forceinline__ void run_own(const BatchArgs &a, const BatchNet<MODE>
     using A = typename Tr<MODE>::A;
     const int lane = tid & 31, warp = tid >> 5;
     auto sync = [] { if (LANES == 32) __syncwarp(); else __syncthreads(); };
-    V v[kOwn], th[kOwn], lk[kOwn], rs[kOwn], ext[kOwn];
-    int rr[kOwn], R[kOwn];
-    unsigned thr[kOwn];
+    V v[SLOTS], th[SLOTS], lk[SLOTS], rs[SLOTS], ext[SLOTS];
+    int rr[SLOTS], R[SLOTS];
+    unsigned thr[SLOTS];
     const long long base = a.rowptr[nb.off];
     const unsigned short *sidx = a.sidx + base;
     const unsigned *sw = a.sw + base;
 #pragma unroll
-    for (int u = 0; u < kOwn; ++u) {
+    for (int u = 0; u < SLOTS; ++u) {
         const int j = u * LANES + tid, g = nb.off + j;
         thr[u] = 0;
         v[u] = th[u] = lk[u] = rs[u] = 0;
@@ -235,7 +238,7 @@ __device__ __forceinline__ void run_own(const BatchArgs &a, const BatchNet<MODE>
     auto prepare = [&](int t) {
         const bool events = t < a.ev_nsteps && a.ev_off[t] < a.ev_off[t + 1];
 #pragma unroll
-        for (int u = 0; u < kOwn; ++u) {
+        for (int u = 0; u < SLOTS; ++u) {
             const int j = u * LANES + tid;
             V x = 0;
             if (events && j < nb.n) {
@@ -260,18 +263,18 @@ __device__ __forceinline__ void run_own(const BatchArgs &a, const BatchNet<MODE>
         int *count = cnt + (s & 1);
         A *slot = ring + (size_t)cur * nb.n;
         unsigned *rrow = a.raster + (size_t)at * a.total_words + nb.woff;
-        A raw[kOwn];
+        A raw[SLOTS];
         unsigned fired = 0;
 #pragma unroll
-        for (int u = 0; u < kOwn; ++u) {
+        for (int u = 0; u < SLOTS; ++u) {
             const int j = u * LANES + tid;
             raw[u] = j < nb.n ? (global_ring ? __ldcg(slot + j) : slot[j]) : (A)0;
         }
-        // the rules of all kOwn neurons first, then their ballots: a neuron past
+        // the rules of all SLOTS neurons first, then their ballots: a neuron past
         // the network's end (no input, no draw, threshold 0) takes its turn too,
         // so that no branch parts one neuron's chain from the next
 #pragma unroll
-        for (int u = 0; u < kOwn; ++u) {
+        for (int u = 0; u < SLOTS; ++u) {
             const V acc = own_from_acc<MODE>(raw[u]);
             bool fire;
             if constexpr (MODE == SN_F32)
@@ -283,7 +286,7 @@ __device__ __forceinline__ void run_own(const BatchArgs &a, const BatchNet<MODE>
         }
         int own = 0;                                       // spikers of the warp
 #pragma unroll
-        for (int u = 0; u < kOwn; ++u) {
+        for (int u = 0; u < SLOTS; ++u) {
             const unsigned ball = __ballot_sync(0xffffffffu, (fired >> u) & 1u);
             const int wb = u * LANES + warp * 32;
             if (lane == 0 && wb < nb.n) rrow[wb >> 5] = ball;
@@ -296,7 +299,7 @@ __device__ __forceinline__ void run_own(const BatchArgs &a, const BatchNet<MODE>
                 first = __shfl_sync(0xffffffffu, first, 0);
             }
 #pragma unroll
-            for (int u = 0; u < kOwn; ++u) {
+            for (int u = 0; u < SLOTS; ++u) {
                 const bool fire = (fired >> u) & 1u;
                 const unsigned ball = __ballot_sync(0xffffffffu, fire);
                 if (fire) list[first + __popc(ball & ((1u << lane) - 1u))] = rows[u * LANES + tid];
@@ -349,7 +352,7 @@ __device__ __forceinline__ void run_own(const BatchArgs &a, const BatchNet<MODE>
         at = at + 1 < a.cap ? at + 1 : 0;
     }
 #pragma unroll
-    for (int u = 0; u < kOwn; ++u) {
+    for (int u = 0; u < SLOTS; ++u) {
         const int j = u * LANES + tid;
         if (j < nb.n) {
             ((V *)a.V)[nb.off + j] = v[u];
@@ -396,9 +399,15 @@ __global__ void __launch_bounds__(kBatchBlock, 2) batch_kernel(BatchArgs a) {
         if (OWN && threadIdx.x < 2) s_own[threadIdx.x] = 0;
         __syncthreads();
         if constexpr (OWN)
-            run_own<MODE, kBatchBlock>(a, nb, ring, !in_smem, threadIdx.x, (int2 *)lists,
-                                       (int2 *)lists + kOwn * kBatchBlock, s_own, my_spikes, my_events,
-                                       overflow);
+        {
+            int2 *list = (int2 *)lists, *rows = list + kOwn * kBatchBlock;
+            if (nb.n <= kBatchBlock)
+                run_own<MODE, kBatchBlock, 1>(a, nb, ring, !in_smem, threadIdx.x, list, rows, s_own, my_spikes,
+                                              my_events, overflow);
+            else
+                run_own<MODE, kBatchBlock, kOwn>(a, nb, ring, !in_smem, threadIdx.x, list, rows, s_own, my_spikes,
+                                                 my_events, overflow);
+        }
         for (int s = OWN ? a.steps : 0; s < a.steps; ++s) {
             const int t = a.t0 + s;
             const int cur = t % a.D1;
@@ -462,7 +471,7 @@ __global__ void __launch_bounds__(kBatchBlock, 2) batch_kernel(BatchArgs a) {
             for (size_t q = lane; q < ring_elems; q += 32) wring_smem[q] = __ldcg(gring + q);
         __syncwarp();
         if constexpr (OWN)
-            run_own<MODE, 32>(a, nb, ring, !in_smem, lane, (int2 *)wlist, (int2 *)wlist + kOwn * 32, nullptr,
+            run_own<MODE, 32, kOwn>(a, nb, ring, !in_smem, lane, (int2 *)wlist, (int2 *)wlist + kOwn * 32, nullptr,
                               my_spikes, my_events, overflow);
         for (int s = OWN ? a.steps : 0; s < a.steps; ++s) {
             const int t = a.t0 + s;
