@@ -82,14 +82,21 @@ sn_status shared_load_spikes(sn_ctx *c, const uint8_t *in) {
 
 sn_status shared_run(sn_ctx *c, int steps) {
     SharedHostArgs h;
-    h.n = c->n; h.B = c->sh_B; h.t0 = (int)c->step; h.steps = steps; h.cap = c->cap;
+    h.n = c->n; h.B = c->sh_B; h.t0 = (int)c->step; h.cap = c->cap;
     h.A0 = c->sh_A0; h.A1 = c->sh_A1; h.V = (int *)c->V; h.r = c->r;
     h.th = (const int *)c->th; h.lk = (const int *)c->lk; h.rs = (const int *)c->rs; h.R = c->R;
     h.prate = c->prate; h.pamp = (const int *)c->pamp; h.pkey = c->pkeys; h.raster = c->raster; h.bits = c->sh_bits;
     h.ctl = c->ctl;
-    cudaError_t e = c->sh_res ? launch_shared_res(c->sh_tmaps + 256, h, c->stream)
-                              : launch_shared(c->sh_tmaps, h, c->sh_grid, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "shared dense launch");
+    // a launch counts the K blocks that a block of threads takes in 32 bits (which
+    // stage, and whether it is free yet): longer runs are several launches
+    const long long tiles = (long long)(h.B / 128) * (h.n / 128);
+    const long long per_step = (h.n / 128) * (c->sh_res ? 1 : (tiles + c->sh_grid - 1) / c->sh_grid);
+    for (int left = steps; left > 0; left -= h.steps, h.t0 += h.steps) {
+        h.steps = (int)std::min<long long>(left, std::max(1ll, (1ll << 31) / per_step));
+        cudaError_t e = c->sh_res ? launch_shared_res(c->sh_tmaps + 256, h, c->stream)
+                                  : launch_shared(c->sh_tmaps, h, c->sh_grid, c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "shared dense launch");
+    }
     return SN_OK;
 }
 
