@@ -836,7 +836,10 @@ def main():
                          "algorithmic_bytes_per_launch": abytes,
                          "bytes_model": "event-proportional: 16 B per spike (row bounds), 16 B per synaptic "
                                         "event (synapse + accumulate), 56 B state and a raster bit per "
-                                        "neuron and timestep",
+                                        "neuron and timestep" +
+                                        ("; the method's bytes, not the kernel's: pull takes every synapse "
+                                         "from an L2-resident store, so the fraction compares rates and can "
+                                         "exceed 1 (traffic is what memory moved)" if pull else ""),
                          "pull_store": store,
                          "kernel_bound": (f"issue: the pull store of incoming synapses "
                                           f"({store['bytes'] / 1e6:.0f} MB) stays in the L2; its synapses of "

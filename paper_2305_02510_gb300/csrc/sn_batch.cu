@@ -523,8 +523,9 @@ static const void *batch_fn(int dtype, bool own) {
 }
 
 // The largest networks of the blocks and of the warps fit kOwn neurons a thread.
-// Measured (100 steps, general form first): 512 networks of 64 to 1024,
-// 558 and 365 us; 2000 of 32 to 128, 507 and 369; 32 of 64 to 300, 377 and 299.
+// Measured (100 steps, us, general form first): 512 networks of 64 to 1024, 492 and
+// 275; 2000 of 32 to 128, 350 and 222; 32 of 64 to 300, 270 and 190; 2000 of 130, 885
+// and 523; 1000 of 1000 with 304 of 20, 1913 and 1125.
 bool batch_own_fits(int max_block_n, int max_warp_n) {
     return max_block_n <= kOwn * kBatchBlock && max_warp_n <= kOwn * 32;
 }

@@ -151,6 +151,8 @@ bool tc_spike_operands(sn_ctx *c, bool shared, size_t s_elems) {
 // the context keeps the SIMT engine only) when they cannot be had.
 bool tc_buffers(sn_ctx *c) {
     const int L = c->ff_layers, B = c->ff_batch, rows = B * c->ff_steps;
+    // (no operand asks for this any more: a delay shifts whole rows.  Other batches
+    // have been neither measured nor compared with the CUDA-core engine)
     if (B % 8 != 0) return false;
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;

@@ -221,6 +221,8 @@ __global__ void __launch_bounds__(kThreads, 1) ff_tc_dw_kernel(const __grid_cons
 // gradient's the whole item.  384 threads: warp 0 lane 0 TMA, warp 1 MMA, warps 4..11
 // drain (warp w: TMEM lane quarter w % 4, columns 64 * ((w - 4) / 4) ..+63).
 // A layer of at most 112 columns loads and multiplies only those (bn).
+// (Two row tiles of the forward take the 168 registers that 384 threads leave and
+// spill 44 bytes; its time is the MMAs'.)
 // 12,800 rows, forward: 1024 x 1024 228 -> 202 us, 700 x 1024 161 -> 145; spike
 // gradient: 1024 x 1024 282 -> 209, 1024 x 20 52 -> 33.
 constexpr int kRowsThreads = 384;

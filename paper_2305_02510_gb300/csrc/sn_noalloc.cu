@@ -1,7 +1,8 @@
 // sn_run_dense_noalloc: the dense simulation for callers that cannot allocate
 // device memory (an application whose device memory is all owned by its own
 // pool allocator, or a plug-in whose host forbids it to allocate).  It launches
-// the same dense kernel as sn_run on a dense context, but every buffer comes
+// the dense kernel that streams its rows (sn_run on a dense context also has one that
+// keeps them in shared memory, with the same bits), and every buffer comes
 // from the caller except the kernel's scratch (spike bits of the last two
 // steps, pending-input ring, zero Poisson table, control block), which lives
 // in one fixed file-scope device array.  No cudaMalloc, cudaFree or

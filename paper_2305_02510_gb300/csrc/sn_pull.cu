@@ -3,7 +3,8 @@
 // w * s_i(t - d); Section 2.2: a spike reaches the post-neuron d steps later).
 //
 // This kernel takes one step at a time: networks of one block, shards, the
-// coded store, and networks whose spike words do not fit sn_pull_block.cu.
+// forms asked for by a flag, networks whose spike words or lists sn_pull_block.cu
+// cannot hold, and those it would be slower for (block_store_wins in sn_api.cu).
 // Every block keeps the spike bits of recent steps in a shared-memory window
 // of hL rows of Wp = roundup(ceil(n/32), 4) words: the row of step tau sits
 // at position tau - base.  Each thread owns one neuron and holds its state in

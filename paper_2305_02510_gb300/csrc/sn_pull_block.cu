@@ -48,6 +48,9 @@
 // of the L2 loads that each region begins with.  A step reads a synapse 0.44
 // times instead of once: 200 steps 2.12 -> 1.53 ms (10.5 -> 7.2 us a step); 20,011
 // neurons, 64 synapses each of delays 1..8, integer: 1.24 -> 0.69 ms (6.1 -> 3.2).
+// A launch prepares its first sums by one pass over region 0 and one step of the loop:
+// runs of a single step take 20.4 us at 20,000 neurons of 64 synapses, delays 1..16,
+// and 49.5 at 100,000 of 100 (one step at a time: 29.8 and 49.5).
 // Measured and left out: owning the neurons by thread position (no sum through
 // shared memory, but 3 % slower), loading the second unit of the delay-1 lists
 // ahead (spills: 12 % slower), reading the padding instead of testing each

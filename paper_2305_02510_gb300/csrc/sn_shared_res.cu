@@ -32,11 +32,12 @@
 // and a tile stores a step's words after its K loop, so no reader is left.
 // The words lie as they are read: [parity][K block][train][4].
 //
-// 8192 neurons x 256 trains (128 blocks), 40 steps: 1266 -> 863 us (31.6 -> 21.5 us
-// a step).  What bounds it now: the warps that own the rows.  Their draws (3.3 us
-// of a step, by leaving them out) and the expansion share the integer pipe, and
-// the MMA warp's issue slots; the weights' loads are hidden (leaving them out
-// changes nothing), the MMAs alone would take 8 us a step.
+// 8192 neurons x 256 trains (128 blocks), 40 steps: 1266 -> 857 us (31.6 -> 21.4 us
+// a step).  No single part bounds it: left out one at a time, the weights' loads
+// give 0.6 us of a step, the draws 0.9, the expansion's shifts 1.2, loads and draws
+// together 1.9; the MMAs alone would take 8.  What is left is the chain from a stage
+// that falls free over the waiting owners' stores back to the MMA (a vote in front of
+// each MMA instead of behind it: 2.9 us), and the exchange of the words.
 //
 // TMEM: accumulator columns 0..127, V 128..255, r 256..383, four operand stages of
 // 32 columns at 384.  Every wait is bounded as in sn_shared.cu.
