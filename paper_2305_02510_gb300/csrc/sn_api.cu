@@ -182,6 +182,9 @@ BlockPlan plan_block_store(const sn_ctx *c, const std::vector<uint2> &syn) {
 //    125 delays 1..4 (1.14) 12.7 | 11.7, 1..6 (0.97) 11.5 | 11.6, 1..16 (0.71) 9.9 | 12.0;
 //    150 delay 1 (1.38) 22.7 | 12.8.  Where the other store does not stay in the L2 either,
 //    r <= 1.2: 200 delays 1..4 (1.12) 22.1 | 25.0, 1..3 (1.28) 26.2 | 25.7.
+//    Delays 1 and 2 alone share nothing between steps and walk two lists: with long ones,
+//    unless a block's stay in its L1, not (10,000 x 1000 25.2 | 24.1, 1000 x 600 15.4 |
+//    15.0; 1000 x 500 7.9 | 12.8, 10,000 x 300 9.8 | 9.8).
 //  - Wide blocks walk slower (64 registers, spills, units of two loads): small stores
 //    (110,000 x 10, delays 1..3, 3.6 | 4.3), delay 1 alone up to a third of the L2
 //    (110,000 x 45 6.6 | 6.8; 140,000 x 60 9.4 | 9.1), and r <= 0.78: 110,000 x 60
@@ -190,7 +193,10 @@ BlockPlan plan_block_store(const sn_ctx *c, const std::vector<uint2> &syn) {
 //    beside a plain store within it: 110,000 x 100 delays 1..12 (0.61) 11.3 | 10.4.
 bool block_store_wins(const sn_ctx *c, const BlockPlan &p, double l2, double old, bool old_coded) {
     const double bytes = (double)p.total * 16.0, reads = p.reads * 16.0;
-    if (c->pull_chunk <= kPullNarrow) return bytes <= 0.72 * l2 || reads <= (old <= 0.8 * l2 ? 1.0 : 1.2) * old;
+    if (c->pull_chunk <= kPullNarrow) {
+        if (c->D == 2 && c->m >= 400ll * c->n && bytes > 140e3 * c->pull_grid) return false;
+        return bytes <= 0.72 * l2 || reads <= (old <= 0.8 * l2 ? 1.0 : 1.2) * old;
+    }
     return bytes <= 0.16 * l2 || (c->D == 1 && bytes <= 0.35 * l2) ||
            (reads <= 0.78 * old && (old_coded || bytes <= 0.85 * l2));
 }
