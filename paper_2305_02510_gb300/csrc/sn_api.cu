@@ -194,7 +194,7 @@ BlockPlan plan_block_store(const sn_ctx *c, const std::vector<uint2> &syn) {
 bool block_store_wins(const sn_ctx *c, const BlockPlan &p, double l2, double old, bool old_coded) {
     const double bytes = (double)p.total * 16.0, reads = p.reads * 16.0;
     if (c->pull_chunk <= kPullNarrow) {
-        if (c->D == 2 && c->m >= 400ll * c->n && bytes > 140e3 * c->pull_grid) return false;
+        if (c->D == 2 && c->m >= 400ll * c->n && bytes > 160e3 * c->pull_grid) return false;
         return bytes <= 0.72 * l2 || reads <= (old <= 0.8 * l2 ? 1.0 : 1.2) * old;
     }
     return bytes <= 0.16 * l2 || (c->D == 1 && bytes <= 0.35 * l2) ||
