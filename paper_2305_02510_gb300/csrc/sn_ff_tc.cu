@@ -272,6 +272,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
     const int items = a.tiles_m * a.tiles_n, steps = 4 * a.kblocks;   // step s: K block s / 4, delay s % 4 + 1
     const int chunk = SG ? steps : 4, chunks = steps / chunk;
     unsigned ua = 0, ub = 0;                       // units this thread has put through (or taken from) the rings
+    unsigned g_chunk = 0;                          // chunks issued, or drained
+    bool live = true;                              // this warp's waits have all seen their phase
 
     if (warp == 0 && lane == 0) {
         const int bytesB = a.bn * 128;
@@ -309,7 +311,6 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
     } else if (warp == 1) {
         const uint32_t idesc = idesc_bf16_f32(kT, a.bn);
         const uint64_t descA = umma_desc_sw128(baseA), descB = umma_desc_sw128(baseB);
-        unsigned g_chunk = 0;
         // barriers are looked at while the MMAs in front of theirs run
         bool seenA = false, seenB = false;
         auto waitA = [&](unsigned u) {
@@ -324,7 +325,6 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
         };
         auto lookA = [&](unsigned u) { seenA = mbar_test_warp(smem_addr(&fullA[u % R::RA]), (u / R::RA) & 1u); };
         auto lookB = [&](unsigned u) { seenB = mbar_test_warp(smem_addr(&fullB[u % R::RB]), (u / R::RB) & 1u); };
-        bool live = true;
         for (int item = blockIdx.x; item < items && live; item += gridDim.x)
             for (int c = 0; c < chunks; ++c, ++g_chunk) {
                 const unsigned buf = g_chunk & 1u, use = g_chunk >> 1;
@@ -383,7 +383,6 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
         if (!live) s_abort = 1;
     } else if (warp >= 4) {
         const int quarter = warp & 3, half = (warp - 4) >> 2;
-        unsigned g_chunk = 0;
         bool ok = true;
         for (int item = blockIdx.x; item < items; item += gridDim.x) {
             const int tm = item % a.tiles_m, tn = item / a.tiles_m;
@@ -443,9 +442,10 @@ __global__ void __launch_bounds__(kRowsThreads, 1) ff_tc_rows_kernel(const __gri
             mbar_drain(smem_addr(&fullB[i % R::RB]), (i / R::RB) & 1u);
     }
     if (warp == 1) {
-        // (every MMA issued, also those of a step that a failed wait cut short)
-        mma_commit(smem_addr(&mmas_done));
-        mbar_drain(smem_addr(&mmas_done), 0);
+        // every MMA issued: up to the last chunk's commit, or those of a step that a
+        // failed wait cut short
+        if (!live) mma_commit(smem_addr(&mmas_done));
+        mbar_drain(smem_addr(live ? &accf[(g_chunk - 1) & 1u] : &mmas_done), live ? ((g_chunk - 1) >> 1) & 1u : 0u);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
