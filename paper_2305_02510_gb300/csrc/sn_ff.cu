@@ -234,13 +234,14 @@ __global__ void __launch_bounds__(kScanBlock) ff_scan_fwd_kernel(const float *__
 // the adjoint: those of segment sg - 1 are copied into the thread's own
 // column of a shared-memory buffer (asynchronous 4-byte copies) while segment
 // sg is computed, and its checkpoint is loaded into registers.
-// With gbf, more threads (columns n .. ldg - 1) zero the padding of its rows: the
+// PAD: more threads (columns n .. ldg - 1) zero the padding of gbf's rows: the
 // buffer is shared by the layers, and what another one left there may be an Inf or a
-// NaN, which the contraction's zero weights would not cancel.  (Tensor maps that end
-// at the true width do the same, but took a step at 700-1024-1024-20 13 us longer.)
+// NaN, which the contraction's zero weights would not cancel.  (A tensor map that ends
+// at the true width does the same, but took a step at 700-1024-1024-20 14 us longer.
+// An instantiation of its own: the branch takes 72 registers instead of 64.)
 constexpr int kBwdBlock = 128;
 
-template <int K>
+template <int K, bool PAD>
 __global__ void __launch_bounds__(kBwdBlock) ff_scan_bwd_kernel(const float *__restrict__ I, int n, int B, int T,
                                    FFNeuron p, const float *__restrict__ vck, const int *__restrict__ rck,
                                    const float *__restrict__ gs, const float *__restrict__ gc,
@@ -248,11 +249,14 @@ __global__ void __launch_bounds__(kBwdBlock) ff_scan_bwd_kernel(const float *__r
     __shared__ float sI[2][K][kBwdBlock], sG[2][K][kBwdBlock];
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (tid >= (long long)B * n) {
-        const int pad = ldg - n;
-        const long long q = tid - (long long)B * n;
-        if (!gbf || q >= (long long)B * pad) return;
-        for (size_t r = (size_t)(q / pad); r < (size_t)2 * T * B; r += B)
-            gbf[r * ldg + n + q % pad] = __float2bfloat16_rn(0.0f);
+        if constexpr (PAD) {
+            // a padding column of one sample's rows
+            const unsigned q = (unsigned)(tid - (long long)B * n), pad = (unsigned)(ldg - n), b = q / pad;
+            if (b >= (unsigned)B) return;
+            __nv_bfloat16 *z = gbf + (size_t)b * ldg + n + (q - b * pad);
+#pragma unroll 1
+            for (int t = 0; t < 2 * T; ++t, z += (size_t)B * ldg) *z = __float2bfloat16_rn(0.0f);
+        }
         return;
     }
     const int b = (int)(tid / n), j = (int)(tid - (long long)(tid / n) * n);
@@ -574,17 +578,18 @@ cudaError_t ff_scan_fwd(const float *I, int n, int B, int T, int k, float theta,
 
 cudaError_t ff_scan_bwd(const float *I, int n, int B, int T, int k, float theta, float leak, float reset,
                         int refractory, float slope, const float *vck, const int *rck, const float *gs,
-                        const float *gc, float *gI, void *gbf, int ldg, cudaStream_t s) {
+                        const float *gc, float *gI, void *gbf, int ldg, bool pad, cudaStream_t s) {
     FFNeuron p{theta, leak, reset, slope, refractory};
-    const long long threads = (long long)B * (gbf ? ldg : n);
+    const long long threads = (long long)B * (pad ? ldg : n);
     const int nb = blocks_for(threads, kBwdBlock);
     __nv_bfloat16 *g2 = (__nv_bfloat16 *)gbf;
+    auto run = [&](auto kernel) { kernel<<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); };
     switch (k) {
-        case 1: ff_scan_bwd_kernel<1><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
-        case 2: ff_scan_bwd_kernel<2><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
-        case 5: ff_scan_bwd_kernel<5><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
-        case 10: ff_scan_bwd_kernel<10><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
-        case 20: ff_scan_bwd_kernel<20><<<nb, kBwdBlock, 0, s>>>(I, n, B, T, p, vck, rck, gs, gc, gI, g2, ldg); break;
+        case 1: pad ? run(ff_scan_bwd_kernel<1, true>) : run(ff_scan_bwd_kernel<1, false>); break;
+        case 2: pad ? run(ff_scan_bwd_kernel<2, true>) : run(ff_scan_bwd_kernel<2, false>); break;
+        case 5: pad ? run(ff_scan_bwd_kernel<5, true>) : run(ff_scan_bwd_kernel<5, false>); break;
+        case 10: pad ? run(ff_scan_bwd_kernel<10, true>) : run(ff_scan_bwd_kernel<10, false>); break;
+        case 20: pad ? run(ff_scan_bwd_kernel<20, true>) : run(ff_scan_bwd_kernel<20, false>); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -398,7 +398,8 @@ sn_status sn_backward(sn_ctx *c, const float *grad_counts, float *const *grad_w,
         if ((e = ff_scan_bwd(I, nout, B, T, c->ff_k, c->ff_theta, c->ff_leak, c->ff_reset, c->ff_refr,
                              c->ff_slope, c->ff_vck[l], c->ff_rck[l], l == L ? nullptr : c->ff_gS,
                              l == L ? grad_counts : nullptr, c->ff_gI, tc ? c->ff_G : nullptr, up(nout, 64),
-                             c->stream)))
+                             // (the first layer's padding is no K of a contraction)
+                             tc && l > 1 && nout % 64 != 0, c->stream)))
             return cuda_fail(c, e, "adjoint recurrence");
         if (tc) {
             sn_status st = tc_weight_grad(c, l, grad_w[l - 1]);

@@ -184,10 +184,11 @@ cudaError_t ff_delay_fwd(const unsigned *sprev, int words_in, const float *W, co
 cudaError_t ff_scan_fwd(const float *I, int n, int B, int T, int k, float theta, float leak, float reset,
                         int refractory, unsigned *S, float *vck, int *rck, float *counts, void *sbf, int ldbf,
                         cudaStream_t s);
-// gI as floats [T*B][n], or (gbf given) as its two BF16 parts [2][T*B][ldg]
+// gI as floats [T*B][n], or (gbf given) as its two BF16 parts [2][T*B][ldg], with pad
+// also zeros in columns n .. ldg - 1
 cudaError_t ff_scan_bwd(const float *I, int n, int B, int T, int k, float theta, float leak, float reset,
                         int refractory, float slope, const float *vck, const int *rck, const float *gs,
-                        const float *gc, float *gI, void *gbf, int ldg, cudaStream_t s);
+                        const float *gc, float *gI, void *gbf, int ldg, bool pad, cudaStream_t s);
 cudaError_t ff_bwd_data(const float *gI, const float *W, const uint8_t *D, int n_in, int n_out, int B, int T,
                         float *gsp, cudaStream_t s);
 cudaError_t ff_dw(const float *gI, const unsigned *sprev, int words_in, const uint8_t *D, int n_in, int n_out,
