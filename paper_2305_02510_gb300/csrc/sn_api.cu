@@ -747,6 +747,7 @@ sn_status sn_create_dense(const sn_config *cfg, const sn_neurons *nr, const floa
     c->block = 256;
     int grid = 0, chunk = 0;
     cudaError_t e = plan_dense(n, &grid, &chunk, force_cpl);
+    if (e == cudaSuccess && grid > 0) e = plan_dense_res(chunk);
     if (e != cudaSuccess) { c->err = std::string("dense executor: ") + cudaGetErrorString(e); return bail(SN_ECUDA); }
     if (grid < 1) {
         c->err = force_cpl ? "the forced column slab gives no co-resident grid for this n"

@@ -403,14 +403,19 @@ size_t dense_tag_bytes(int n) {
     return words > kMaxWords ? 0 : (size_t)2 * words * kDenseTagStride * 8;
 }
 
+cudaError_t plan_dense_res(int chunk) {
+    if (chunk > 128) return cudaSuccess;
+    for (const void *fn : {res_fn(chunk / 32, false, false), res_fn(chunk / 32, false, true), res_fn(chunk / 32, true, false)})
+        if (cudaError_t e = allow_all_smem(fn)) return e;
+    return cudaSuccess;
+}
+
 cudaError_t launch_dense_res(const NetArgs &a, int grid, cudaStream_t s) {
     const bool vec = a.n % 4 == 0 && ((uintptr_t)a.W & 15u) == 0;
     const void *fn = res_fn(a.chunk / 32, a.stdp != 0, vec);
-    cudaError_t e = allow_all_smem(fn);
-    if (e != cudaSuccess) return e;
     if (grid > 1) {
         dense_tag_init_kernel<<<1, 256, 0, s>>>(a.ptag, 2 * a.words * kDenseTagStride);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (cudaError_t e = cudaGetLastError()) return e;
     }
     void *args[] = {(void *)&a};
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kThreads), args, res_smem(a.n, a.chunk, a.stdp != 0), s);

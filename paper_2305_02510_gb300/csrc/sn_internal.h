@@ -238,6 +238,7 @@ constexpr int kDenseResSteps = 4, kDenseResStepsStdp = 12;   // shortest runs th
 constexpr int kDenseTagStride = 16;        // 64-bit words from one spike word of a tagged row to the next
 size_t dense_tag_bytes(int n);             // 0: n never takes it
 bool dense_res_fits(int n, int chunk, int grid, bool stdp, int steps);
+cudaError_t plan_dense_res(int chunk);     // before the first launch
 cudaError_t launch_dense_res(const NetArgs &a, int grid, cudaStream_t s);
 cudaError_t plan_dense(int n, int *grid, int *chunk, int force_cpl = 0);
 // Pull propagation (sn_pull.cu).  plan_pull sets *grid = 0 when the network
