@@ -361,10 +361,12 @@ __device__ __forceinline__ void run_own(const BatchArgs &a, const BatchNet<MODE>
     }
 }
 
-// OWN: every network takes run_own (batch_own_fits); a kernel of its own, because
-// with both forms in one the registers of either spill (136 bytes; networks of
-// 4096 neurons 1.7 times the time).
-template <int MODE, bool OWN>
+// FORM 0: the general form; 1 and 2: every network takes run_own (batch_form), with 2
+// the blocks' networks of one neuron a thread in an instantiation of theirs.  Kernels
+// of their own: with the general form in one the registers of either spill (136 bytes;
+// networks of 4096 neurons 1.7 times the time), and with the one-slot loop in it the
+// others' are about 1 % slower (100 networks of 300 to 1024, 60 steps: 207.5 us and 205.7).
+template <int MODE, int FORM>
 __global__ void __launch_bounds__(kBatchBlock, 2) batch_kernel(BatchArgs a) {
     using A = typename Tr<MODE>::A;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -378,6 +380,7 @@ __global__ void __launch_bounds__(kBatchBlock, 2) batch_kernel(BatchArgs a) {
     // Some blocks, the last ones, take warps' networks from the start: a warp needs
     // as long for one of 128 neurons as a block for one of 1024, and begun after
     // the blocks' queue was empty they were the last 250 us of 480.
+    constexpr bool OWN = FORM != 0;
     const int early = OWN && a.n_cta ? min((a.n_warp + kWarps - 1) / kWarps, (int)gridDim.x / 8) : 0;
     const bool warps_first = (int)(gridDim.x - blockIdx.x) <= early;
     // ---- networks run by the whole block
@@ -401,7 +404,7 @@ __global__ void __launch_bounds__(kBatchBlock, 2) batch_kernel(BatchArgs a) {
         if constexpr (OWN)
         {
             int2 *list = (int2 *)lists, *rows = list + kOwn * kBatchBlock;
-            if (nb.n <= kBatchBlock)
+            if (FORM == 2 && nb.n <= kBatchBlock)
                 run_own<MODE, kBatchBlock, 1>(a, nb, ring, !in_smem, threadIdx.x, list, rows, s_own, my_spikes,
                                               my_events, overflow);
             else
@@ -517,33 +520,37 @@ __global__ void __launch_bounds__(kBatchBlock, 2) batch_kernel(BatchArgs a) {
 
 size_t batch_smem(int ring_smem) { return (size_t)ring_smem + (size_t)kListInts * sizeof(int); }
 
-static const void *batch_fn(int dtype, bool own) {
-    if (own) return dtype == SN_F32 ? (const void *)batch_kernel<SN_F32, true> : (const void *)batch_kernel<SN_I32, true>;
-    return dtype == SN_F32 ? (const void *)batch_kernel<SN_F32, false> : (const void *)batch_kernel<SN_I32, false>;
+static const void *batch_fn(int dtype, int form) {
+    const bool f = dtype == SN_F32;
+    if (form == 2) return f ? (const void *)batch_kernel<SN_F32, 2> : (const void *)batch_kernel<SN_I32, 2>;
+    if (form == 1) return f ? (const void *)batch_kernel<SN_F32, 1> : (const void *)batch_kernel<SN_I32, 1>;
+    return f ? (const void *)batch_kernel<SN_F32, 0> : (const void *)batch_kernel<SN_I32, 0>;
 }
 
-// The largest networks of the blocks and of the warps fit kOwn neurons a thread.
+// run_own where the largest networks of the blocks and of the warps fit kOwn neurons a
+// thread (sizes of the blocks' networks: 0, 0 when there are none).
 // Measured (100 steps, us, general form first): 512 networks of 64 to 1024, 492 and
 // 275; 2000 of 32 to 128, 350 and 222; 32 of 64 to 300, 270 and 190; 2000 of 130, 885
 // and 523; 1000 of 1000 with 304 of 20, 1913 and 1125.
-bool batch_own_fits(int max_block_n, int max_warp_n) {
-    return max_block_n <= kOwn * kBatchBlock && max_warp_n <= kOwn * 32;
+int batch_form(int min_block_n, int max_block_n, int max_warp_n) {
+    if (max_block_n > kOwn * kBatchBlock || max_warp_n > kOwn * 32) return 0;
+    return min_block_n > 0 && min_block_n <= kBatchBlock ? 2 : 1;
 }
 
-cudaError_t batch_kernel_node(int dtype, bool own, void **fn) {
-    *fn = (void *)batch_fn(dtype, own);
+cudaError_t batch_kernel_node(int dtype, int form, void **fn) {
+    *fn = (void *)batch_fn(dtype, form);
     return cudaSuccess;
 }
 
-cudaError_t max_grid_batch(int dtype, bool own, int ring_smem, int *grid) {
+cudaError_t max_grid_batch(int dtype, int form, int ring_smem, int *grid) {
     int dev = 0, sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const size_t smem = batch_smem(ring_smem);
-    if ((e = allow_all_smem(batch_fn(dtype, own))) != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_fn(dtype, own), kBatchBlock, smem);
+    if ((e = allow_all_smem(batch_fn(dtype, form))) != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_fn(dtype, form), kBatchBlock, smem);
     if (e != cudaSuccess) return e;
     *grid = per * sms;
     return cudaSuccess;

@@ -26,12 +26,9 @@ static sn_status batch_upload_orders(sn_ctx *c) {
     std::sort(small.begin(), small.end(), by_size);
     c->n_cta = (int)big.size();
     c->n_warp = (int)small.size();
-    auto largest = [&](const std::vector<int> &v) {
-        int n = 0;
-        for (int b : v) n = std::max(n, c->h_net_n[b]);
-        return n;
-    };
-    c->batch_own = batch_own_fits(largest(big), largest(small));
+    // (both lists are sorted, the largest first)
+    c->batch_form = batch_form(big.empty() ? 0 : c->h_net_n[big.back()], big.empty() ? 0 : c->h_net_n[big.front()],
+                               small.empty() ? 0 : c->h_net_n[small.front()]);
     if (!big.empty()) SN_CUDA(c, cudaMemcpy(c->cta_order, big.data(), big.size() * 4, cudaMemcpyHostToDevice));
     if (!small.empty()) SN_CUDA(c, cudaMemcpy(c->warp_order, small.data(), small.size() * 4, cudaMemcpyHostToDevice));
     return SN_OK;
@@ -65,7 +62,7 @@ static BatchArgs batch_args(sn_ctx *c, int steps) {
 sn_status batch_run(sn_ctx *c, int steps) {
     BatchArgs a = batch_args(c, steps);
     void *fn = nullptr;
-    batch_kernel_node(c->dtype, c->batch_own, &fn);
+    batch_kernel_node(c->dtype, c->batch_form, &fn);
     void *args[] = {(void *)&a};
     cudaKernelNodeParams kp;
     memset(&kp, 0, sizeof(kp));
@@ -96,7 +93,7 @@ sn_status batch_run(sn_ctx *c, int steps) {
 
 static sn_status batch_size_grid(sn_ctx *c) {
     int g = 0;
-    cudaError_t e = max_grid_batch(c->dtype, c->batch_own, c->ring_smem, &g);
+    cudaError_t e = max_grid_batch(c->dtype, c->batch_form, c->ring_smem, &g);
     if (e != cudaSuccess) return cuda_fail(c, e, "batch occupancy");
     if (g < 1) return fail(c, SN_EUNSUPPORTED, "batched kernel cannot be resident with this shared memory");
     c->batch_grid = g;

@@ -93,7 +93,7 @@ struct sn_ctx {
     unsigned short *sidx = nullptr;
     unsigned *sw = nullptr;
     int n_cta = 0, n_warp = 0;
-    bool batch_own = false;              // every network fits the form that keeps its state in registers
+    int batch_form = 0;                  // 1, 2: every network fits the form that keeps its state in registers
     int warp_max_n = 128, ring_smem = 96 * 1024, batch_grid = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t graph_exec = nullptr;

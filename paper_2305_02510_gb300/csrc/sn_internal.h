@@ -148,9 +148,9 @@ constexpr int kBatchBlock = 256;
 constexpr int kBatchMaxN = 4096;      // largest network of a batched context
 constexpr int kBatchMaxDelay = 16;
 
-bool batch_own_fits(int max_block_n, int max_warp_n);
-cudaError_t batch_kernel_node(int dtype, bool own, void **fn);
-cudaError_t max_grid_batch(int dtype, bool own, int ring_smem, int *grid);
+int batch_form(int min_block_n, int max_block_n, int max_warp_n);
+cudaError_t batch_kernel_node(int dtype, int form, void **fn);
+cudaError_t max_grid_batch(int dtype, int form, int ring_smem, int *grid);
 size_t batch_smem(int ring_smem);
 
 // Shared dense network on tensor cores: sn_shared.cu, and sn_shared_res.cu when
